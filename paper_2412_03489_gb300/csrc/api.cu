@@ -568,6 +568,8 @@ hr_status hr_create_scene(const hr_scene_desc* d, hr_scene* out) {
         if (e != cudaSuccess) return bail(e, "target render");
     }
     if (sc.kind == HR_SCENE_REVOLVE3D) revolve_tile_t2(sc, s->stream);
+    if (sc.kind == HR_SCENE_TRIS2D && (e = tris2d_prepare_target(sc, s->stream)) != cudaSuccess)
+        return bail(e, "target tiles");
     if ((sc.kind == HR_SCENE_DISC2D || sc.kind == HR_SCENE_BOXES2D) &&
         (e = disc_prepare_target(sc, s->stream)) != cudaSuccess)
         return bail(e, "target bits");
@@ -582,7 +584,7 @@ hr_status hr_destroy_scene(hr_scene s) {
     DevScene& sc = s->sc;
     if (s->stream) cudaStreamSynchronize(s->stream);
     cudaFree(sc.target); cudaFree(sc.verts); cudaFree(sc.tris); cudaFree(sc.tnrm); cudaFree(sc.tile_t2);
-    cudaFree(sc.raw); cudaFree(sc.pidx); cudaFree(sc.qA); cudaFree(sc.qb); cudaFree(sc.rv_stats);
+    cudaFree(sc.raw); cudaFree(sc.pidx); cudaFree(sc.target4); cudaFree(sc.qA); cudaFree(sc.qb); cudaFree(sc.rv_stats);
     cudaFree(sc.pt_stats); cudaFree(sc.tbits); cudaFree(sc.trowpop);
     s->ws.release_all();
     for (cudaEvent_t& e : s->ev)

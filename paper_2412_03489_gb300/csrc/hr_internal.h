@@ -173,6 +173,7 @@ struct DevScene {
     float* raw = nullptr;         // [n_tris][9]
     int32_t* pidx = nullptr;      // [n]
     int n_tris = 0;
+    float* target4 = nullptr;     // [tiles][32][4] target and its squares in 8x4 tile order
     // ptbox
     int32_t qaxis[13] = {};
     float qgeom[13][5] = {};
@@ -205,6 +206,7 @@ bool revolve_layout(DevScene& sc, int max_smem, int smem_per_sm);
 int revolve_tiles(const DevScene& sc);
 void revolve_prepare(DevScene& sc, cudaStream_t s);   // normals, kernel attributes
 void revolve_tile_t2(DevScene& sc, cudaStream_t s);   // after the target exists
+cudaError_t tris2d_prepare_target(DevScene& sc, cudaStream_t s);   // after the target exists: sc.target4
 // disc and squares scenes, after the target exists: sc.tbits, sc.trowpop and sc.tbinary
 cudaError_t disc_prepare_target(DevScene& sc, cudaStream_t s);
 
