@@ -537,6 +537,7 @@ hr_status hr_create_scene(const hr_scene_desc* d, hr_scene* out) {
                 for (int c = 0; c < 3; ++c) { sc.sc_[i][c] = d->sph_center[3 * i + c]; sc.salb[i][c] = d->sph_albedo[3 * i + c]; }
                 sc.sr[i] = d->sph_radius[i];
             }
+            if ((e = ptbox_prepare()) != cudaSuccess) return bail(e, "kernel attributes");
             sc.light_half = d->light_half; sc.cam_z = d->cam_z; sc.tan_half = d->tan_half; sc.pix_scale = d->pix_scale;
             for (int c = 0; c < 3; ++c) sc.emission[c] = d->emission[c];
             sc.spp = d->spp; sc.target_spp = d->target_spp; sc.depth = d->depth; sc.scene_seed = d->seed;

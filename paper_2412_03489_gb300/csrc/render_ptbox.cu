@@ -17,6 +17,7 @@
 // try; blocks 1..3 hold tries 1..6; a cosine-weighted direction comes from a
 // unit-disc point (rejection from the square) lifted to the hemisphere.
 #include <cmath>
+#include <cooperative_groups.h>
 
 #include "hr_device.cuh"
 #include "hr_internal.h"
@@ -421,6 +422,611 @@ ptbox_kernel(PtArgs A, RenderBatch b, const float* __restrict__ img_params, uint
     }
 }
 
+// ---------------------------------------------------------------------------
+// Both legs of an antithetic pair by one CTA.  The legs share their path
+// random numbers and differ in the light's and sphere 0's centre only, so
+// their paths are the same rays until one of them meets the light or
+// sphere 0.  A lane follows the common path of its pixel sample for the legs
+// still on it (`mask`): the random words, the rays, the tests of the twelve
+// quads and spheres 1 and 2 and the surface are formed once, the light,
+// sphere 0 and the shadow ray once per leg.  A leg that meets the light ends.
+// A leg that meets sphere 0 while the other stays on the common path goes to the
+// warp's queue, whose entries are finished 32 at a time, one leg per lane (all
+// pending ones before the warp's next sample of a pixel, so that a leg adds its
+// contributions in vertex and sample order).
+//
+// Every value is formed by the operations of `radiance`, and the closest hit is
+// the least (t, primitive index) of the accepted ones in either order of tests,
+// so losses are the same bits as one render per CTA gives.
+//
+// Bound by issue and its latencies (71 % of slots busy; the loop's code is about
+// as large as the instruction cache holds, so each part of it exists once and
+// queued legs run the same loop as camera paths: with separate code for them
+// 18.0 ms against 14.2 per 2,048 renders of 128x128, 4 spp).  Of the 4,700
+// instructions per pair and path sample 2,000 are shadow rays, 740 queued legs; two
+// single renders take 6,150.  8,192 renders of 128x128, 4 spp: 54.6 ms with one
+// render per CTA, 41.6 with pairs.  Four CTAs of 64 registers per SM: 4,864
+// renders in 27.7 ms, three of 80 registers 31.0.
+// ---------------------------------------------------------------------------
+constexpr int kQueue = 64;     // 31 left over + one push per lane
+constexpr int kQueueWords = 10;
+constexpr int kPairWarps = kThreads / 32;
+
+struct PairLeg {
+    float4 light;              // lo_u, lo_v, hi_u, hi_v
+    float4 sph;                // sphere 0: centre, r^2
+    float plane;               // light plane y
+    float area;
+    int light_inside;
+    int pad;
+};
+struct PairShared {
+    float4 rect[12];           // quads: lo_u, lo_v, hi_u, hi_v
+    float plane[12];
+    float4 sph[2];             // spheres 1, 2
+    uint4 keys[5];             // Philox round keys
+    float alb[16][3];
+    float isr[3];
+    float em[3];
+    float box_lo[3], box_hi[3];
+    int wall_lo[3], wall_hi[3];
+    PairLeg leg[2];
+    float p[2][8];
+    float part[2][kPairWarps];
+};
+template <int kSlots>   // pixels per lane between two ends of the queue
+struct PairWarp {
+    float L[kSlots][6][32];    // radiance sums of the slots' pixels: 3 leg + channel
+    float q[kQueueWords][kQueue];
+    float acc[2][32];          // loss sums of the lanes, by leg
+};
+
+struct Hit {
+    float t;
+    int prim;
+};
+
+// philox10 with the key schedule of the pair's seed (ten (k0, k1), read as five float4)
+__device__ __forceinline__ u32x4 philox_keyed(const PairShared& S, uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3) {
+#pragma unroll
+    for (int r = 0; r < 10; r += 2) {
+        const uint4 k = S.keys[r >> 1];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint64_t pa = (uint64_t)0xD2511F53u * c0, pb = (uint64_t)0xCD9E8D57u * c2;
+            const uint32_t a = (uint32_t)pa, ha = (uint32_t)(pa >> 32), b = (uint32_t)pb, hb = (uint32_t)(pb >> 32);
+            const uint32_t n0 = hb ^ c1 ^ (h ? k.z : k.x), n2 = ha ^ c3 ^ (h ? k.w : k.y);
+            c0 = n0; c1 = b; c2 = n2; c3 = a;
+        }
+    }
+    return {c0, c1, c2, c3};
+}
+
+__device__ __forceinline__ void quad_hit(float4 R, float plane, int q, int a, const float o[3], const float d[3],
+                                         const float inv[3], Hit& h) {
+    const int u = a == 0 ? 1 : 0, v = a == 2 ? 1 : 2;
+    // d_a = 0: t is infinite or NaN and the last compare rejects it
+    const float t = __fmul_rn(__fsub_rn(plane, o[a]), inv[a]);
+    const float hu = __fmaf_rn(t, d[u], o[u]);
+    const float hv = __fmaf_rn(t, d[v], o[v]);
+    const bool ok = t > 0.0f && !(hu < R.x || hu > R.z || hv < R.y || hv > R.w) && t < h.t;
+    h.t = ok ? t : h.t;
+    h.prim = ok ? q : h.prim;
+}
+
+// |o - c|^2 - r^2 of a sphere: the part of its test that depends on the origin only
+__device__ __forceinline__ float sphere_cc(float4 sp, const float o[3]) {
+    const float oc[3] = {__fsub_rn(o[0], sp.x), __fsub_rn(o[1], sp.y), __fsub_rn(o[2], sp.z)};
+    return __fsub_rn(dot3(oc, oc), sp.w);
+}
+
+// Distance of the sphere's first root > 0 (see intersect), -1 when it is not
+// hit.  With the origin outside (cc > 0) and the sphere behind (b >= 0)
+// neither root is positive: disc = fma(b, b, -cc) <= RN(b^2), so its square
+// root is at most b.  The roots are formed only when some lane of the warp
+// needs them.
+__device__ __forceinline__ float sphere_t(float4 sp, float cc, const float o[3], const float d[3], bool live) {
+    const float oc[3] = {__fsub_rn(o[0], sp.x), __fsub_rn(o[1], sp.y), __fsub_rn(o[2], sp.z)};
+    const float b = dot3(oc, d);
+    const float disc = __fmaf_rn(b, b, -cc);
+    const bool on = live && disc >= 0.0f && (b < 0.0f || cc <= 0.0f);
+    float t = -1.0f;
+    if (__any_sync(0xffffffffu, on)) {
+        const float sq = __fsqrt_rn(fmaxf(disc, 0.0f));
+        const float t0 = __fsub_rn(-b, sq);
+        if (on) t = t0 > 0.0f ? t0 : __fsub_rn(sq, b);
+    }
+    return t;
+}
+
+// A ray's origin, with what the tests of several rays from it share.
+struct Origin {
+    float o[3];
+    float cc[2];   // sphere_cc of spheres 1, 2
+    bool in;       // inside the walls
+};
+
+__device__ __forceinline__ bool in_box(const PairShared& S, const float o[3]) {
+    return o[0] >= S.box_lo[0] && o[0] <= S.box_hi[0] && o[1] >= S.box_lo[1] && o[1] <= S.box_hi[1] &&
+           o[2] >= S.box_lo[2] && o[2] <= S.box_hi[2];
+}
+
+// wall q's distance where its hit lies in the rectangle, else -1 (any axis)
+__device__ __noinline__ float any_axis_t(const PairShared& S, int q, float ox, float oy, float oz, float dx, float dy,
+                                         float dz) {
+    const int a = q >> 1;
+    const float oa = a == 0 ? ox : (a == 1 ? oy : oz), da = a == 0 ? dx : (a == 1 ? dy : dz);
+    const float ou = a == 0 ? oy : ox, du = a == 0 ? dy : dx;
+    const float ov = a == 2 ? oy : oz, dv = a == 2 ? dy : dz;
+    const float t = __fmul_rn(__fsub_rn(S.plane[q], oa), __frcp_rn(da));
+    const float hu = __fmaf_rn(t, du, ou), hv = __fmaf_rn(t, dv, ov);
+    const float4 R = S.rect[q];
+    return t > 0.0f && !(hu < R.x || hu > R.z || hv < R.y || hv > R.w) && t < INFINITY ? t : -1.0f;
+}
+
+// closest of the primitives both legs share (all but the light and sphere 0)
+__device__ __forceinline__ Hit closest_shared(const PairShared& S, const Origin& O, const float d[3],
+                                              const float inv[3], bool live) {
+    const float* o = O.o;
+    Hit h{INFINITY, -1};
+    if (O.in) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const int q = d[a] > 0.0f ? S.wall_hi[a] : S.wall_lo[a];
+            quad_hit(S.rect[q], S.plane[q], q, a, o, d, inv, h);
+        }
+    } else {
+        for (int q = 0; q < 6; ++q) {   // rare: not unrolled, to keep the code small
+            const float t = any_axis_t(S, q, o[0], o[1], o[2], d[0], d[1], d[2]);
+            if (t > 0.0f && t < h.t) { h.t = t; h.prim = q; }
+        }
+    }
+#pragma unroll
+    for (int q = 6; q < 12; ++q) quad_hit(S.rect[q], S.plane[q], q, (q - 6) >> 1, o, d, inv, h);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const float t = sphere_t(S.sph[i], O.cc[i], o, d, live);
+        const bool ok = t > 0.0f && t < h.t;
+        h.t = ok ? t : h.t;
+        h.prim = ok ? 14 + i : h.prim;
+    }
+    return h;
+}
+
+// adds one leg's light and sphere 0; equal distances go to the lower index
+__device__ __forceinline__ void add_leg(const PairLeg& G, const float o[3], const float d[3], const float inv[3],
+                                        bool live, Hit& h) {
+    const float t = __fmul_rn(__fsub_rn(G.plane, o[1]), inv[1]);
+    const float hu = __fmaf_rn(t, d[0], o[0]);
+    const float hv = __fmaf_rn(t, d[2], o[2]);
+    const float4 R = G.light;
+    if (t > 0.0f && !(hu < R.x || hu > R.z || hv < R.y || hv > R.w) && t < INFINITY &&
+        (t < h.t || (t == h.t && h.prim > kLight))) {
+        h.t = t;
+        h.prim = kLight;
+    }
+    const float ts = sphere_t(G.sph, sphere_cc(G.sph, o), o, d, live);
+    if (ts > 0.0f && (ts < h.t || (ts == h.t && h.prim > 13))) {
+        h.t = ts;
+        h.prim = 13;
+    }
+}
+
+// Is the light the closest primitive along a shadow ray?  The light's
+// distance first, then any primitive that takes its place: a quad (lower
+// index) at most as far, a sphere (higher index) nearer.
+__device__ __forceinline__ bool light_seen(const PairShared& S, const PairLeg& G, const Origin& O, const float d[3],
+                                           bool live) {
+    const float* o = O.o;
+    const float inv1 = __frcp_rn(d[1]);
+    const float tl = __fmul_rn(__fsub_rn(G.plane, o[1]), inv1);
+    const float lu = __fmaf_rn(tl, d[0], o[0]);
+    const float lv = __fmaf_rn(tl, d[2], o[2]);
+    const float4 R = G.light;
+    bool seen = live && tl > 0.0f && !(lu < R.x || lu > R.z || lv < R.y || lv > R.w) && tl < INFINITY;
+    auto blocks = [&](float4 Q, float plane, int a, const float* inv) {
+        const int u = a == 0 ? 1 : 0, v = a == 2 ? 1 : 2;
+        const float t = __fmul_rn(__fsub_rn(plane, o[a]), inv[a]);
+        const float hu = __fmaf_rn(t, d[u], o[u]);
+        const float hv = __fmaf_rn(t, d[v], o[v]);
+        return t > 0.0f && !(hu < Q.x || hu > Q.z || hv < Q.y || hv > Q.w) && t <= tl;
+    };
+    if (!__any_sync(0xffffffffu, seen)) return false;
+    if (!(O.in && G.light_inside)) {
+        for (int q = 0; q < 6; ++q) {   // rare: not unrolled, the walls behind an inside origin are rejected too
+            const float t = any_axis_t(S, q, o[0], o[1], o[2], d[0], d[1], d[2]);
+            seen = seen && !(t > 0.0f && t <= tl);
+        }
+    }
+    __syncwarp();
+    {
+        const float inv[3] = {__frcp_rn(d[0]), inv1, __frcp_rn(d[2])};
+#pragma unroll
+        for (int q = 6; q < 12; ++q) seen = seen && !blocks(S.rect[q], S.plane[q], (q - 6) >> 1, inv);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const float4 sp = i == 0 ? G.sph : S.sph[i - 1];
+        const float t = sphere_t(sp, i == 0 ? sphere_cc(sp, o) : O.cc[i - 1], o, d, seen);
+        seen = seen && !(t > 0.0f && t < tl);
+    }
+    return seen;
+}
+
+// surface at the hit: normal against the ray and the offset origin
+__device__ __forceinline__ void surface(const PairShared& S, const PairLeg& G, int prim, const float x[3],
+                                        const float d[3], float n[3], float o2[3]) {
+    if (prim < 12) {
+        const int a = prim < 6 ? prim >> 1 : (prim - 6) >> 1;
+        const float da = a == 0 ? d[0] : (a == 1 ? d[1] : d[2]);
+        const float s = da > 0.0f ? -1.0f : 1.0f;
+        n[0] = a == 0 ? s : 0.0f;
+        n[1] = a == 1 ? s : 0.0f;
+        n[2] = a == 2 ? s : 0.0f;
+    } else {
+        const float4 sp = prim == 13 ? G.sph : S.sph[prim - 14];
+        const float isr = S.isr[prim - 13];
+        n[0] = __fmul_rn(__fsub_rn(x[0], sp.x), isr);
+        n[1] = __fmul_rn(__fsub_rn(x[1], sp.y), isr);
+        n[2] = __fmul_rn(__fsub_rn(x[2], sp.z), isr);
+        if (dot3(n, d) > 0.0f) { n[0] = -n[0]; n[1] = -n[1]; n[2] = -n[2]; }
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) o2[c] = __fmaf_rn(n[c], 1e-4f, x[c]);
+}
+
+// next-event estimation of one leg: adds to its radiance sums L[c][0];
+// power: throughput times albedo times emission
+__device__ __forceinline__ void add_light(const PairShared& S, const PairLeg& G, bool live, const u32x4& w0,
+                                          const float n[3], const Origin& O, const float power[3], float (*L)[32]) {
+    const float* o2 = O.o;
+    const float4 R = G.light;
+    const float ly[3] = {__fmaf_rn(u24f(w0.x), __fsub_rn(R.z, R.x), R.x), G.plane,
+                         __fmaf_rn(u24f(w0.y), __fsub_rn(R.w, R.y), R.y)};
+    const float wv[3] = {__fsub_rn(ly[0], o2[0]), __fsub_rn(ly[1], o2[1]), __fsub_rn(ly[2], o2[2])};
+    const float dist2 = dot3(wv, wv);
+    const float idist = __frcp_rn(__fsqrt_rn(dist2));
+    const float om[3] = {__fmul_rn(wv[0], idist), __fmul_rn(wv[1], idist), __fmul_rn(wv[2], idist)};
+    const float cosx = dot3(n, om);
+    const float cosl = om[1];
+    live = live && cosx > 0.0f && cosl > 0.0f;
+    if (light_seen(S, G, O, om, live)) {
+        const float geo = __fmul_rn(__fmul_rn(__fdiv_rn(__fmul_rn(cosx, cosl), dist2), G.area), kInvPi);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) L[c][0] = __fmaf_rn(power[c], geo, L[c][0]);
+    }
+    __syncwarp();
+}
+
+// cosine-weighted continuation around n (see radiance)
+__device__ __forceinline__ void next_direction(const PairShared& S, uint32_t idx, uint32_t cbase, uint32_t c2,
+                                               uint32_t request, const u32x4& w0, const float n[3], float nd[3]) {
+    float a = 0.0f, b = 0.0f;
+    {
+        float ta = __fmaf_rn(u24f(w0.z), 2.0f, -1.0f), tb = __fmaf_rn(u24f(w0.w), 2.0f, -1.0f);
+        bool found = __fmaf_rn(ta, ta, __fmul_rn(tb, tb)) < 1.0f;
+        if (found) { a = ta; b = tb; }
+        for (uint32_t blk = 1; blk <= 3 && !found; ++blk) {
+            const u32x4 wb = philox_keyed(S, idx, cbase | blk, c2, request);
+            ta = __fmaf_rn(u24f(wb.x), 2.0f, -1.0f);
+            tb = __fmaf_rn(u24f(wb.y), 2.0f, -1.0f);
+            found = __fmaf_rn(ta, ta, __fmul_rn(tb, tb)) < 1.0f;
+            if (!found) {
+                ta = __fmaf_rn(u24f(wb.z), 2.0f, -1.0f);
+                tb = __fmaf_rn(u24f(wb.w), 2.0f, -1.0f);
+                found = __fmaf_rn(ta, ta, __fmul_rn(tb, tb)) < 1.0f;
+            }
+            if (found) { a = ta; b = tb; }
+        }
+    }
+    __syncwarp();
+    const float r2 = __fmaf_rn(a, a, __fmul_rn(b, b));
+    const float cz = __fsqrt_rn(__fsub_rn(1.0f, r2));
+    const float sg = copysignf(1.0f, n[2]);
+    const float aa = __fdiv_rn(-1.0f, __fadd_rn(sg, n[2]));
+    const float bb = __fmul_rn(__fmul_rn(n[0], n[1]), aa);
+    const float t1[3] = {__fmaf_rn(__fmul_rn(sg, __fmul_rn(n[0], n[0])), aa, 1.0f), __fmul_rn(sg, bb),
+                         -__fmul_rn(sg, n[0])};
+    const float t2[3] = {bb, __fmaf_rn(__fmul_rn(n[1], n[1]), aa, sg), -n[1]};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) nd[c] = __fmaf_rn(cz, n[c], __fmaf_rn(b, t2[c], __fmul_rn(a, t1[c])));
+}
+
+// What the paths of one pair have in common.
+struct PairRng {
+    uint32_t request, c2, k;
+};
+
+__device__ void load_pair(const PtArgs& A, PairShared& S) {
+    const int t = threadIdx.x;
+    if (t < 12) {
+        S.rect[t] = make_float4(A.qgeom[t][1], A.qgeom[t][2], A.qgeom[t][3], A.qgeom[t][4]);
+        S.plane[t] = A.qgeom[t][0];
+        for (int c = 0; c < 3; ++c) S.alb[t][c] = A.qalb[t][c];
+    } else if (t == 12) {
+        S.alb[12][0] = S.alb[12][1] = S.alb[12][2] = 0.0f;
+    } else if (t < 16) {
+        const int i = t - 13;
+        if (i > 0) S.sph[i - 1] = make_float4(A.sc[i][0], A.sc[i][1], A.sc[i][2], __fmul_rn(A.sr[i], A.sr[i]));
+        for (int c = 0; c < 3; ++c) S.alb[t][c] = A.salb[i][c];
+        S.isr[i] = __frcp_rn(A.sr[i]);
+        S.em[i] = A.em[i];
+        // wall planes of axis i (quads 2 i, 2 i + 1)
+        const float p0 = A.qgeom[2 * i][0], p1 = A.qgeom[2 * i + 1][0];
+        S.box_lo[i] = fminf(p0, p1);
+        S.box_hi[i] = fmaxf(p0, p1);
+        S.wall_lo[i] = p0 <= p1 ? 2 * i : 2 * i + 1;
+        S.wall_hi[i] = p0 <= p1 ? 2 * i + 1 : 2 * i;
+    } else if (t < 18) {
+        PairLeg& G = S.leg[t - 16];
+        const float* p = S.p[t - 16];
+        G.light = make_float4(__fsub_rn(p[0], A.light_half), __fsub_rn(p[2], A.light_half),
+                              __fadd_rn(p[0], A.light_half), __fadd_rn(p[2], A.light_half));
+        G.plane = p[1];
+        G.area = __fmul_rn(__fsub_rn(G.light.z, G.light.x), __fsub_rn(G.light.w, G.light.y));
+        G.sph = make_float4(p[3], p[4], p[5], __fmul_rn(A.sr[0], A.sr[0]));
+        const float lmin[3] = {G.light.x, G.plane, G.light.y}, lmax[3] = {G.light.z, G.plane, G.light.w};
+        bool in = true;
+        for (int a = 0; a < 3; ++a) {
+            const float p0 = A.qgeom[2 * a][0], p1 = A.qgeom[2 * a + 1][0];
+            in = in && lmin[a] >= fminf(p0, p1) + kWallMargin && lmax[a] <= fmaxf(p0, p1) - kWallMargin;
+        }
+        G.light_inside = in ? 1 : 0;
+    }
+}
+
+// kSplit: the CTAs of a cluster render one pair, each a round of kSlots x 256
+// pixels at a time; rank 0 adds up their pixels in order.
+template <int kMinBlocks, int kSlots, bool kSplit>
+__global__ void __launch_bounds__(kThreads, kMinBlocks) ptbox_pair_kernel(PtArgs A, RenderBatch b) {
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    PairShared& S = *reinterpret_cast<PairShared*>(s_dyn);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    PairWarp<kSlots>& Q = reinterpret_cast<PairWarp<kSlots>*>(s_dyn + ((sizeof(PairShared) + 15) & ~size_t(15)))[warp];
+    cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    const int parts = kSplit ? (int)cluster.num_blocks() : 1, rank = kSplit ? (int)cluster.block_rank() : 0;
+    const int m = 2 * ((int)blockIdx.x / parts);
+    PairRng rng;
+    {
+        const Pert pt = resolve(b, m);
+        if (tid == 32) {
+            uint32_t k0 = (uint32_t)pt.seed, k1 = (uint32_t)(pt.seed >> 32);
+            for (int r = 0; r < 5; ++r) {
+                S.keys[r] = make_uint4(k0, k1, k0 + 0x9E3779B9u, k1 + 0xBB67AE85u);
+                k0 += 2u * 0x9E3779B9u;
+                k1 += 2u * 0xBB67AE85u;
+            }
+        }
+        rng.request = pt.request;
+        const uint2 mt = *pt.meta;
+        rng.c2 = (TAG_PATH << 24) | (mt.x & 0xFFFFFFu);
+        rng.k = mt.y;
+        if (tid < 16) {
+            const int leg = tid >> 3, j = tid & 7;
+            const Pert pl = resolve(b, m + leg);
+            if (j < 6) S.p[leg][j] = __fadd_rn(pl.theta[j], pl.tau[j]);
+        }
+    }
+    __syncthreads();
+    load_pair(A, S);
+    __syncthreads();
+    const int spp = A.spp, depth = A.depth, npx = A.W * A.H;
+    const float inv_spp = 1.0f / (float)spp;
+    Q.acc[0][lane] = Q.acc[1][lane] = 0.0f;
+    const uint64_t w_recip = ((1ull << 40) + (uint64_t)A.W - 1) / (uint64_t)A.W;
+    for (int first = 0; first < npx; first += parts * kSlots * kThreads) {
+        const int px0 = first + rank * kSlots * kThreads + warp * 32;
+#pragma unroll
+        for (int i = 0; i < kSlots * 6; ++i) (&Q.L[0][0][0])[i * 32 + lane] = 0.0f;
+        __syncwarp();
+        int s = 0, slot = 0, queued = 0;
+        const int slots = max(0, min(kSlots, (npx - px0 + kThreads - 1) / kThreads));
+        while (slots > 0) {
+            // the next batch of the warp: 32 queued legs (fewer at a sample's
+            // end), or the camera paths of the next slot's pixels
+            const bool finish = queued >= 32 || (slot == slots && queued > 0);
+            if (!finish && slot == slots) {
+                slot = 0;
+                if (++s == spp) break;
+            }
+            uint32_t mask;          // legs on this lane's path
+            int leg = 0, vert = 1;  // leg: the one leg of a queued path
+            int prim = 13;
+            float t = 0.0f;
+            Origin O;
+            float* o = O.o;
+            float d[3], beta[3];
+            uint32_t idx;
+            float (*L)[32];
+            if (finish) {
+                const int n = min(queued, 32);
+                queued -= n;
+                const int e = queued + (lane < n ? lane : 0);
+                // the hit on sphere 0 is stored as the origin, t = 0
+#pragma unroll
+                for (int c = 0; c < 3; ++c) { o[c] = Q.q[c][e]; d[c] = Q.q[3 + c][e]; beta[c] = Q.q[6 + c][e]; }
+                const uint32_t meta = __float_as_uint(Q.q[9][e]);   // lane | slot << 8 | leg << 16 | vertex << 24
+                const int from = (int)((meta >> 8) & 0xFFu), src = (int)(meta & 31u);
+                leg = (int)((meta >> 16) & 1u);
+                vert = (int)(meta >> 24);
+                mask = lane < n ? 1u << leg : 0u;
+                idx = (uint32_t)((px0 + from * kThreads + src) * spp + s);
+                L = reinterpret_cast<float (*)[32]>(&Q.L[from][0][src]);
+                __syncwarp();
+            } else {
+                const int px = px0 + slot * kThreads + lane;
+                mask = px < npx ? 3u : 0u;
+                const int y = (int)(((uint64_t)(uint32_t)px * w_recip) >> 40), xp = px - y * A.W;
+                idx = (uint32_t)(px * spp + s);
+                const u32x4 wj = philox_keyed(S, idx, rng.k << 8, rng.c2, rng.request);
+                const float fx = __fadd_rn((float)xp, u24f(wj.x));
+                const float fy = __fadd_rn((float)y, u24f(wj.y));
+                d[0] = __fmaf_rn(fx, A.pix_scale, -A.tan_half);
+                d[1] = __fmaf_rn(-fy, A.pix_scale, A.tan_half);
+                d[2] = -1.0f;
+                const float il = __frcp_rn(__fsqrt_rn(dot3(d, d)));
+                d[0] = __fmul_rn(d[0], il); d[1] = __fmul_rn(d[1], il); d[2] = __fmul_rn(d[2], il);
+                o[0] = 0.0f; o[1] = 0.0f; o[2] = A.cam_z;
+                beta[0] = beta[1] = beta[2] = 1.0f;
+                L = reinterpret_cast<float (*)[32]>(&Q.L[slot][0][lane]);
+            }
+            O.in = in_box(S, o);
+            O.cc[0] = sphere_cc(S.sph[0], o);
+            O.cc[1] = sphere_cc(S.sph[1], o);
+            const int legs = finish ? 1 : 2;   // a queued path has its own leg, a camera path both
+            bool resume = finish;              // queued paths start at their hit
+#pragma unroll 1
+            for (;;) {
+                if (!resume) {
+                    // the common ray's closest hit, then each leg's
+                    const float inv[3] = {__frcp_rn(d[0]), __frcp_rn(d[1]), __frcp_rn(d[2])};
+                    const Hit hs = closest_shared(S, O, d, inv, mask != 0u);
+                    uint32_t on_sphere = 0u;
+                    float t_sph = 0.0f, t_sph1 = 0.0f;
+#pragma unroll 1
+                    for (int j = 0; j < legs; ++j) {
+                        const int l = finish ? leg : j;
+                        const uint32_t bit = 1u << l;
+                        Hit h = hs;
+                        add_leg(S.leg[l], o, d, inv, (mask & bit) != 0u, h);
+                        if (mask & bit) {
+                            if (h.prim == 13) {
+                                on_sphere |= bit;
+                                t_sph1 = h.t;
+                                if (on_sphere == bit) t_sph = h.t;
+                            } else if (h.prim < 0 || h.prim == kLight) {
+                                if (vert == 1 && h.prim == kLight && d[1] > 0.0f)
+                                    for (int c = 0; c < 3; ++c) L[3 * l + c][0] = __fadd_rn(L[3 * l + c][0], S.em[c]);
+                                mask &= ~bit;
+                            }
+                        }
+                    }
+                    // the lane goes on with the legs on the common surface, or
+                    // with one leg on sphere 0 when there are none; the other
+                    // leg on sphere 0 is queued
+                    prim = hs.prim;
+                    t = hs.t;
+                    uint32_t push = on_sphere;
+                    if (on_sphere != 0u && on_sphere == mask) {
+                        prim = 13;
+                        t = t_sph;   // the first leg's
+                        if (!finish) leg = (on_sphere & 1u) ? 0 : 1;
+                        push = on_sphere & ~(1u << leg);
+                    }
+                    if (!finish) {
+                        mask &= ~push;
+                        const unsigned pushers = __ballot_sync(0xffffffffu, push != 0u);
+                        if (pushers) {
+                            if (push) {
+                                const int e = queued + __popc(pushers & ((1u << lane) - 1u));
+#pragma unroll
+                                for (int c = 0; c < 3; ++c) {
+                                    Q.q[c][e] = __fmaf_rn(t_sph1, d[c], o[c]);
+                                    Q.q[3 + c][e] = d[c];
+                                    Q.q[6 + c][e] = beta[c];
+                                }
+                                Q.q[9][e] = __uint_as_float((uint32_t)lane | ((uint32_t)slot << 8) |
+                                                            ((push >> 1) << 16) | ((uint32_t)vert << 24));
+                            }
+                            queued += __popc(pushers);
+                            __syncwarp();
+                        }
+                    }
+                    if (!__any_sync(0xffffffffu, mask != 0u)) break;
+                    if (mask == 0u) prim = 0;
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) o[c] = __fmaf_rn(t, d[c], o[c]);
+                }
+                resume = false;
+                float n[3], x[3] = {o[0], o[1], o[2]};
+                surface(S, S.leg[leg], prim, x, d, n, o);
+                O.in = in_box(S, o);
+                O.cc[0] = sphere_cc(S.sph[0], o);
+                O.cc[1] = sphere_cc(S.sph[1], o);
+                float power[3];
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    beta[c] = __fmul_rn(beta[c], S.alb[prim][c]);
+                    power[c] = __fmul_rn(beta[c], S.em[c]);
+                }
+                const uint32_t cbase = (rng.k << 8) | ((uint32_t)vert << 4);
+                const u32x4 w0 = philox_keyed(S, idx, cbase, rng.c2, rng.request);
+#pragma unroll 1
+                for (int j = 0; j < legs; ++j) {
+                    const int l = finish ? leg : j;
+                    add_light(S, S.leg[l], ((mask >> l) & 1u) != 0u, w0, n, O, power, L + 3 * l);
+                }
+                if (vert >= depth) mask = 0u;
+                if (!__any_sync(0xffffffffu, mask != 0u)) break;
+                next_direction(S, idx, cbase, rng.c2, rng.request, w0, n, d);
+                ++vert;
+            }
+            __syncwarp();
+            if (!finish) ++slot;
+        }
+#pragma unroll
+        for (int slot = 0; slot < kSlots; ++slot) {
+            const int px = px0 + slot * kThreads + lane;
+            if (px < npx) {
+                const float* tg = A.target + 3 * (size_t)px;
+                const float g0 = tg[0], g1 = tg[1], g2 = tg[2];
+#pragma unroll
+                for (int l = 0; l < 2; ++l) {
+                    const float d0 = __fmaf_rn(Q.L[slot][3 * l][lane], inv_spp, -g0);
+                    const float d1 = __fmaf_rn(Q.L[slot][3 * l + 1][lane], inv_spp, -g1);
+                    const float d2 = __fmaf_rn(Q.L[slot][3 * l + 2][lane], inv_spp, -g2);
+                    const float v = __fmaf_rn(d2, d2, __fmaf_rn(d0, d0, __fmul_rn(d1, d1)));
+                    if (kSplit) Q.L[slot][3 * l][lane] = v;
+                    else Q.acc[l][lane] = __fadd_rn(Q.acc[l][lane], v);
+                }
+            }
+        }
+        __syncwarp();
+        if (kSplit) {
+            cluster.sync();
+            if (rank == 0) {
+                for (int q = 0; q < parts; ++q) {
+                    const PairWarp<kSlots>* R = cluster.map_shared_rank(&Q, q);
+                    const int qx0 = first + q * kSlots * kThreads + warp * 32 + lane;
+#pragma unroll
+                    for (int slot = 0; slot < kSlots; ++slot)
+                        if (qx0 + slot * kThreads < npx)
+                            for (int l = 0; l < 2; ++l) Q.acc[l][lane] = __fadd_rn(Q.acc[l][lane], R->L[slot][3 * l][lane]);
+                }
+            }
+            cluster.sync();
+        }
+    }
+    if (kSplit && rank != 0) return;
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {
+        const float v = warp_sum(Q.acc[l][lane]);
+        if (lane == 0) S.part[l][warp] = v;
+    }
+    __syncthreads();
+    if (tid < 2) {
+        float v = 0.0f;
+        for (int w = 0; w < kPairWarps; ++w) v += S.part[tid][w];
+        *resolve(b, m + tid).loss = v / (float)(npx * 3);
+    }
+}
+
+template <int kSlots>
+constexpr size_t pair_smem() {
+    return ((sizeof(PairShared) + 15) & ~size_t(15)) + kPairWarps * sizeof(PairWarp<kSlots>);
+}
+constexpr int kWhole = 5;   // slots of a CTA that renders a whole pair
+
+// every two items 2 i, 2 i + 1 of the launch are the legs of one pair
+bool in_pairs(const RenderBatch& b) {
+    if (b.M & 1) return false;
+    if (b.table_rows <= 0) return (b.per_row & 1) == 0;
+    for (int r = 0; r < b.table_rows; ++r)
+        if ((b.rows[r].start & 1) || (b.rows[r].m_begin & 1)) return false;
+    return true;
+}
+
 PtArgs make_args(const DevScene& sc) {
     PtArgs a;
     for (int q = 0; q < 13; ++q) {
@@ -448,6 +1054,65 @@ bool canonical_axes(const DevScene& sc) {
     return true;
 }
 
+template <int kSlots>
+void launch_parts(const PtArgs& a, const RenderBatch& b, int parts, cudaStream_t s) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)parts;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3((unsigned)(b.M / 2) * (unsigned)parts);
+    c.blockDim = dim3(kThreads);
+    c.dynamicSmemBytes = pair_smem<kSlots>();
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    cudaLaunchKernelEx(&c, ptbox_pair_kernel<4, kSlots, true>, a, b);
+}
+
+// CTAs that share one pair of renders (1: none) and the pixels per lane of their
+// rounds.  Both kernels compute the same bits; the lines come from timing them
+// (GB300, 152 SMs; us, one render per CTA / pairs as chosen here):
+//   8x8 to 24x24          one render: 46 / 101 at 16x16, 4 spp, M = 64
+//   32x32, 4 spp          M 64: 158 / 105; 256: 189 / 212; 1,024: 496 / 557; 4,096: 1,754 / 1,561
+//   48x48, 2 spp          M 64: 179 / 116; 256: 210 / 265; 1,024: 556 / 552; 4,096: 1,971 / 1,739
+//   64x64, 2 spp          M 256: 364 / 308; 1,024: 975 / 896; 4,096: 3,459 / 3,137
+//   128x128, 4 spp        M 64: 2,363 / 750; 1,024: 7,606 / 6,547; 4,096: 27,182 / 23,903
+// A pair's lane has a longer serial chain (both legs' shadow rays) than a
+// render's, so pairs need images of some size, and below 64x64 either few
+// renders, each spread over a cluster, or enough to fill the GPU.
+struct PairShape {
+    int parts = 0, slots = 4;   // parts 0: one render per CTA
+};
+PairShape pair_shape(int npx, int pairs, int sms) {
+    PairShape p;
+    if (npx < 1024) return p;
+    if (npx < 4096 && 2 * pairs > sms && 2 * pairs < 13 * sms) return p;
+    p.parts = 1;
+    // several waves of CTAs even out the end: split while a part keeps two rounds
+    while (p.parts < 8 && pairs * p.parts < 16 * sms && 4096 * p.parts <= npx) p.parts *= 2;
+    // fewer CTAs than the GPU holds: split on, down to 256 pixels a part
+    while (p.parts < 8 && pairs * p.parts < 4 * sms && kThreads * p.parts < npx) p.parts *= 2;
+    while (p.slots > 1 && p.slots * kThreads * p.parts >= 2 * npx) p.slots /= 2;
+    while (p.slots > 1 && p.slots * kThreads * (p.parts / 2) >= npx) p.slots /= 2;
+    return p;
+}
+
+void launch_pairs(int variant, const PtArgs& a, const RenderBatch& b, const PairShape& p, cudaStream_t s) {
+    const int pairs = b.M / 2;
+    if (p.parts > 1) {
+        if (p.slots == 4) launch_parts<4>(a, b, p.parts, s);
+        else if (p.slots == 2) launch_parts<2>(a, b, p.parts, s);
+        else launch_parts<1>(a, b, p.parts, s);
+        return;
+    }
+    switch (variant) {
+        case 1: ptbox_pair_kernel<3, kWhole, false><<<pairs, kThreads, pair_smem<kWhole>(), s>>>(a, b); break;
+        case 2: ptbox_pair_kernel<2, kWhole, false><<<pairs, kThreads, pair_smem<kWhole>(), s>>>(a, b); break;
+        default: ptbox_pair_kernel<4, kWhole, false><<<pairs, kThreads, pair_smem<kWhole>(), s>>>(a, b); break;
+    }
+}
+
 template <bool kCanon>
 void launch_loss(const DevScene& sc, const RenderBatch& b, cudaStream_t s) {
     const PtArgs a = make_args(sc);
@@ -455,10 +1120,20 @@ void launch_loss(const DevScene& sc, const RenderBatch& b, cudaStream_t s) {
         ptbox_kernel<false, 3, kCanon, true><<<b.M, kThreads, 0, s>>>(a, b, nullptr, 0, 0, 0, 0, 0, 0, nullptr);
         return;
     }
-    switch (sc.render_variant) {
-        case 1: ptbox_kernel<false, 2, kCanon><<<b.M, kThreads, 0, s>>>(a, b, nullptr, 0, 0, 0, 0, 0, 0, nullptr); break;
-        case 2: ptbox_kernel<false, 4, kCanon><<<b.M, kThreads, 0, s>>>(a, b, nullptr, 0, 0, 0, 0, 0, 0, nullptr); break;
-        default: ptbox_kernel<false, 3, kCanon><<<b.M, kThreads, 0, s>>>(a, b, nullptr, 0, 0, 0, 0, 0, 0, nullptr); break;
+    const PairShape p = kCanon && in_pairs(b) ? pair_shape(sc.W * sc.H, b.M / 2, num_sms()) : PairShape{};
+    if (p.parts > 0) {
+        launch_pairs(sc.render_variant, a, b, p, s);
+        return;
+    }
+    // variant 0: as many resident CTAs per SM as the launch has, 2 to 4 (fewer
+    // leave each its registers; 24x24, M = 64: 31 us with 2, 35 with 3, 38 with 4;
+    // M = 1,024: 101 with 3, 89 with 4)
+    const int shape = sc.render_variant == 1 ? 3 : sc.render_variant == 2 ? 2
+                      : b.M <= 2 * num_sms() ? 2 : b.M <= 3 * num_sms() ? 3 : 4;
+    switch (shape) {
+        case 2: ptbox_kernel<false, 2, kCanon><<<b.M, kThreads, 0, s>>>(a, b, nullptr, 0, 0, 0, 0, 0, 0, nullptr); break;
+        case 3: ptbox_kernel<false, 3, kCanon><<<b.M, kThreads, 0, s>>>(a, b, nullptr, 0, 0, 0, 0, 0, 0, nullptr); break;
+        default: ptbox_kernel<false, 4, kCanon><<<b.M, kThreads, 0, s>>>(a, b, nullptr, 0, 0, 0, 0, 0, 0, nullptr); break;
     }
 }
 
@@ -466,11 +1141,21 @@ void launch_loss(const DevScene& sc, const RenderBatch& b, cudaStream_t s) {
 
 // Launch-shape variants (autotuner): the same 256-thread layout and
 // arithmetic, different register caps through the minimum number of resident
-// CTAs per SM (3, 2, 4), so the choice never changes a result.  Scenes with
-// the procedural box's quad layout use the compile-time-axis intersection.
+// CTAs per SM (4 or by the launch's size, 3, 2), so the choice never changes a
+// result.  Scenes with the procedural box's quad layout use the
+// compile-time-axis intersection, and the pair kernel where it is faster.
 void launch_ptbox_loss(const DevScene& sc, const RenderBatch& b, cudaStream_t s) {
     if (canonical_axes(sc)) launch_loss<true>(sc, b, s);
     else launch_loss<false>(sc, b, s);
+}
+
+cudaError_t ptbox_prepare() {
+    cudaError_t e = cudaSuccess;
+    for (auto k : {ptbox_pair_kernel<2, kWhole, false>, ptbox_pair_kernel<3, kWhole, false>,
+                   ptbox_pair_kernel<4, kWhole, false>})
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pair_smem<kWhole>());
+    return e;
 }
 
 void launch_ptbox_image(const DevScene& sc, const float* params, uint64_t seed, uint32_t request, uint32_t sub,
