@@ -276,7 +276,7 @@ hr_status run_estimate(hr_scene_s* s, int quantity, const double* h_theta, const
     fa.hessian = quantity == HR_HESSIAN;
     fa.inv2P = 1.0 / (double)M;
     fa.out_flat = (double*)ws.flat.ptr;
-    fa.out_scale = (double*)ws.scale.ptr;
+    fa.out_scale = h_out && o->out_scale ? (double*)ws.scale.ptr : nullptr;
     fa.out_full = quantity == HR_HESSIAN ? (d_out ? d_out : (double*)ws.full.ptr) : nullptr;
     if (quantity != HR_HESSIAN && d_out) fa.out_flat = d_out;
     launch_finalize(fa, stream);

@@ -52,7 +52,7 @@ constexpr int kInlineGroups = 4;
 void launch_sample(const SampleArgs& a, int n_groups, int max_P, cudaStream_t s);
 
 // g[b][e] = 1/Mg sum of w[m][e] loss[m] over rows [b per_inst, b per_inst + Mg)
-// (Kahan FP32 chunks, FP64 tree); grid (n, B)
+// (Kahan FP32 chunks, FP64 tree)
 void launch_grad_reduce(const float* w, const float* loss, int n, int per_inst, int Mg, int B, double* g,
                         cudaStream_t s);
 
@@ -65,9 +65,13 @@ struct FinalizeArgs {
     int32_t elementwise;  // element e sums rows [e*2P, (e+1)*2P), else [0, 2P)
     int32_t hessian;      // also write the symmetric n x n matrix
     double inv2P;
-    double* out_flat;     // [E]
-    double* out_scale;    // [E] or null
+    double* out_flat;     // [E] ([batches][E])
+    double* out_scale;    // [E] or null (not formed)
     double* out_full;     // [n][n] or null
+    // several sums of the same shape: batch b's rows start at b row_stride
+    int32_t batches;      // 0 or 1: one
+    int32_t row_stride;
+    int32_t divide;       // 1: divide by pairs2 instead of multiplying by inv2P
 };
 void launch_finalize(const FinalizeArgs& a, cudaStream_t s);
 

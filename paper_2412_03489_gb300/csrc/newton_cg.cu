@@ -33,25 +33,6 @@ __global__ void theta32_kernel(const double* th, float* th32, int count) {
     if (i < count) th32[i] = __double2float_rn(th[i]);
 }
 
-// g[b][e] = 1/Mg sum over the instance's gradient rows of w[m][e] loss[m]
-__global__ void __launch_bounds__(256) grad_reduce_kernel(const float* w, const float* loss, int n, int per_inst,
-                                                          int Mg, double* g) {
-    __shared__ double sh[256];
-    const int e = blockIdx.x, b = blockIdx.y;
-    const int m0 = b * per_inst;
-    const int chunk = (Mg + 255) / 256;
-    const int beg = m0 + threadIdx.x * chunk, end = min(m0 + Mg, beg + chunk);
-    Kahan k;
-    for (int m = beg; m < end; ++m) k.add(__fmul_rn(w[(size_t)m * n + e], loss[m]));
-    sh[threadIdx.x] = (double)k.s - (double)k.c;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) g[b * n + e] = sh[0] / (double)Mg;
-}
-
 struct CgArgs {
     int n, per_inst, Mg, Mh, K;
     double sigma, lambda_rel, delta;
@@ -143,7 +124,17 @@ __global__ void advance_step_kernel(int32_t* step) { *step += 1; }
 
 void launch_grad_reduce(const float* w, const float* loss, int n, int per_inst, int Mg, int B, double* g,
                         cudaStream_t s) {
-    grad_reduce_kernel<<<dim3(n, B), 256, 0, s>>>(w, loss, n, per_inst, Mg, g);
+    FinalizeArgs a{};
+    a.w = w;
+    a.loss = loss;
+    a.E = n;
+    a.n = n;
+    a.pairs2 = Mg;
+    a.divide = 1;
+    a.out_flat = g;
+    a.batches = B;
+    a.row_stride = per_inst;
+    launch_finalize(a, s);
 }
 
 }  // namespace hr

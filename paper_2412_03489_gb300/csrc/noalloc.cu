@@ -175,7 +175,7 @@ extern "C" hr_status hr_estimate_dev_noalloc(hr_scene s, int32_t quantity, const
     fa.hessian = quantity == HR_HESSIAN;
     fa.inv2P = 1.0 / (double)M;
     fa.out_flat = quantity == HR_HESSIAN ? reinterpret_cast<double*>(base + off_flat) : d_out;
-    fa.out_scale = reinterpret_cast<double*>(base + off_scale);
+    fa.out_scale = nullptr;   // not an output of this form
     fa.out_full = quantity == HR_HESSIAN ? d_out : nullptr;
     launch_finalize(fa, stream);
     const cudaError_t e = cudaGetLastError();

@@ -1,7 +1,7 @@
 // Device code of the perturbation sampler (Sec. 3.2-3.5), shared by the
 // sampler kernel (sample.cu) and the persistent serving kernel (queue.cu):
 // FP64 lobe inverses, the mixture densities and the weights, and one pair
-// leg's draw.
+// leg's draw by one thread (the persistent kernel's form).
 #pragma once
 #include <cmath>
 
@@ -178,7 +178,12 @@ __device__ __forceinline__ double recip_mixture(double S) {
 }
 
 // S(tau): n^2 q(tau) / N(tau) for the Hessian mixture, O(n) via
-// sum_{i != j} |t_i t_j| = (sum |t_i|)^2 - sum t_i^2.
+// sum_{i != j} |t_i t_j| = (sum |t_i|)^2 - sum t_i^2; from sd = sum |t_i^2 - s^2|,
+// sa = sum |t_i|, sq = sum t_i^2.
+__device__ __forceinline__ double hess_density(double sd, double sa, double sq, const Lobes& L) {
+    const double off = sa * sa - sq;
+    return (sd * L.is4 * L.iZd + (off > 0.0 ? off : 0.0) * L.is4 * L.iZo) * L.inv_n2;
+}
 __device__ double hess_mixture(const float* t, int n, const Lobes& L) {
     double sd = 0.0, sa = 0.0, sq = 0.0;
     for (int d = 0; d < n; ++d) {
@@ -187,8 +192,52 @@ __device__ double hess_mixture(const float* t, int n, const Lobes& L) {
         sa += fabs(x);
         sq += x * x;
     }
-    const double off = sa * sa - sq;
-    return (sd * L.is4 * L.iZd + (off > 0.0 ? off : 0.0) * L.is4 * L.iZo) * L.inv_n2;
+    return hess_density(sd, sa, sq, L);
+}
+
+// S of the gradient mixture
+__device__ double grad_mixture(const float* t, int n, const Lobes& L) {
+    double S = 0.0;
+    for (int d = 0; d < n; ++d) S += fabs((double)t[d] * L.is2);
+    return S * L.iZg * L.inv_n;
+}
+
+// sum_d t_d v_d in dim order
+__device__ double dot_dims(const float* t, const double* v, int n) {
+    double tv = 0.0;
+    for (int d = 0; d < n; ++d) tv += (double)t[d] * v[d];
+    return tv;
+}
+
+// weight of an element-wise HVP draw of row i: h_i^v / q_i of the row mixture
+__device__ double row_weight(const double* v, int n, int i, const Lobes& L, const float* t) {
+    const double ti = (double)t[i];
+    double hv = 0.0, den = 0.0, tot = 0.0;
+    for (int b = 0; b < n; ++b) {
+        const double c = (b == i) ? (ti * ti - L.s2) * L.is4 : ti * (double)t[b] * L.is4;
+        hv += c * v[b];
+        den += fabs(v[b]) * fabs(c);
+        tot += fabs(v[b]) * (b == i ? L.Zd : L.Zo);
+    }
+    return den > 0.0 ? hv * tot / den : 0.0;
+}
+
+// component j of row i with probability |v_j| Z_ij / sum_l |v_l| Z_il (cumulative
+// sums in index order), from one Philox word
+__device__ int row_component(const double* v, int n, int i, const Lobes& L, uint32_t word) {
+    double tot = 0.0;
+    for (int l = 0; l < n; ++l) tot += fabs(v[l]) * (l == i ? L.Zd : L.Zo);
+    const double u = u01d(word) * tot;
+    double acc = 0.0;
+    int j = i, last = i;
+    bool found = false;
+    for (int l = 0; l < n; ++l) {
+        const double p = fabs(v[l]) * (l == i ? L.Zd : L.Zo);
+        if (p > 0.0) last = l;
+        acc += p;
+        if (!found && p > 0.0 && u < acc) { j = l; found = true; }
+    }
+    return found ? j : last;
 }
 
 // Args: SampleArgs, or any type with the fields read here and in sample_leg
@@ -217,24 +266,13 @@ __device__ void write_weights(const Args& a, const Lobes& L, const SampleGroup& 
                     wm[e] = (float)((i == jj) ? (ti * ti - s2) * is4 : ti * (double)t[jj] * is4);
             }
         } else {
-            double tv = 0.0;
-            for (int d = 0; d < n; ++d) tv += (double)t[d] * a.v[d];
+            const double tv = dot_dims(t, a.v, n);
             for (int kk = 0; kk < n; ++kk) wm[kk] = (float)((double)t[kk] * tv * is4 - a.v[kk] * is2);
         }
         return;
     }
     if (G.quantity == 4) {
-        // element-wise HVP, row i: h_i^v / q_i of the row mixture
-        const int i = G.comp_i;
-        const double ti = (double)t[i];
-        double hv = 0.0, den = 0.0, tot = 0.0;
-        for (int b = 0; b < n; ++b) {
-            const double c = (b == i) ? (ti * ti - s2) * is4 : ti * (double)t[b] * is4;
-            hv += c * a.v[b];
-            den += fabs(a.v[b]) * fabs(c);
-            tot += fabs(a.v[b]) * (b == i ? L.Zd : L.Zo);
-        }
-        wm[i] = (float)(den > 0.0 ? hv * tot / den : 0.0);
+        wm[G.comp_i] = (float)row_weight(a.v, n, G.comp_i, L, t);
         return;
     }
     if (G.comp_i >= 0) {
@@ -247,9 +285,7 @@ __device__ void write_weights(const Args& a, const Lobes& L, const SampleGroup& 
         return;
     }
     if (G.quantity == 0) {
-        double S = 0.0;
-        for (int d = 0; d < n; ++d) S += fabs((double)t[d] * is2);
-        S = S * L.iZg * L.inv_n;
+        const double S = grad_mixture(t, n, L);
         const double iS = S > 0.0 ? recip_mixture(S) : 0.0;
         for (int d = 0; d < n; ++d) wm[d] = (float)(((double)t[d] * is2) * iS);
         return;
@@ -267,8 +303,7 @@ __device__ void write_weights(const Args& a, const Lobes& L, const SampleGroup& 
             }
         }
     } else {
-        double tv = 0.0;
-        for (int d = 0; d < n; ++d) tv += (double)t[d] * a.v[d];
+        const double tv = dot_dims(t, a.v, n);
         for (int k = 0; k < n; ++k) {
             const double hv = (double)t[k] * tv * is4 - a.v[k] * is2;
             wm[k] = (float)(hv * iS);
@@ -277,8 +312,7 @@ __device__ void write_weights(const Args& a, const Lobes& L, const SampleGroup& 
 }
 
 // One leg (0: + lobe, 1: - lobe) of antithetic pair k of group G: its
-// perturbation, path key and weights (Sec. 3.2-3.5).  Called by the sampler
-// kernel (two threads per pair) and by the persistent serving kernel.
+// perturbation, path key and weights (Sec. 3.2-3.5).
 template <class Args>
 __device__ __forceinline__ void sample_leg(const Args& a, const SampleGroup& G, const Lobes& L, int k, int leg) {
     const int n = a.n;
@@ -290,23 +324,8 @@ __device__ __forceinline__ void sample_leg(const Args& a, const SampleGroup& G, 
     if (G.comp_i == -3) {
         i = -1; j = -1;            // no importance sampling: every dim Gaussian
     } else if (G.comp_i >= 0 && G.comp_j == -2) {
-        // element-wise HVP: component j of row i with probability
-        // |v_j| Z_ij / sum_l |v_l| Z_il (cumulative sums in index order)
-        i = G.comp_i;
-        double tot = 0.0;
-        for (int l = 0; l < n; ++l) tot += fabs(a.v[l]) * (l == i ? L.Zd : L.Zo);
-        const double u = u01d(w0.x) * tot;
-        double acc = 0.0;
-        j = i;
-        int last = i;
-        bool found = false;
-        for (int l = 0; l < n; ++l) {
-            const double p = fabs(a.v[l]) * (l == i ? L.Zd : L.Zo);
-            if (p > 0.0) last = l;
-            acc += p;
-            if (!found && p > 0.0 && u < acc) { j = l; found = true; }
-        }
-        if (!found) j = last;
+        i = G.comp_i;   // element-wise HVP: a component of row i
+        j = row_component(a.v, n, i, L, w0.x);
     } else if (G.comp_i >= 0) {
         i = G.comp_i;
         j = G.lobe == 0 ? G.comp_i : G.comp_j;
