@@ -127,17 +127,24 @@ __device__ __forceinline__ float disc_rows(const float* __restrict__ target, int
 //     (|cy| + r) H 2^-22 + 1 rows, so every such row lies inside the
 //     real-arithmetic band (cy -+ r) H - 1/2 widened by 2 + (|cy| + r) H 2^-20
 //     rows; the rows [y0, y1) of that band are the only ones tested.
-// A row's span ends are found with the exact test itself, in a window of four
-// columns around the real-arithmetic ends cx -+ sqrt(r^2 - dy^2); an end
-// outside the window falls back to a binary search on the same predicate.  Rows outside [y0, y1) differ from the target in its set pixels
-// (a prefix sum of the rows' popcounts); a row inside differs in
-// popc(target bits XOR span bits) over its words (an empty span when its
-// dy^2 >= r^2).
+// An end is the real-arithmetic one, cx -+ sqrt(r^2 - dy^2), when the exact test
+// holds on its inner side and fails on its outer side: a change of the test
+// inside one interval's ends is that end.  Otherwise (an end within rounding of
+// a pixel centre, a row whose interval may be empty) exact_span finds both.
+// With the target's ones counted by column (pre[y][x] ones in the first x
+// pixels of row y) the mismatches are the target's ones plus, for every row, the
+// interval's length less twice the ones inside it: two loads a row, whatever
+// the width.
+// Bound by the latency of a warp's loads and tests (a row is about 45
+// instructions).  Render stage in us, with windows of four tests per end and
+// the row's words XORed, and now: 16,384 discs of 333x250 32.4, 16.7; 256 of
+// 512x512 16.0, 10.6; 16,384 of 512x512 107, 22.9; 64x64: 7.8, 7.8 (launch).
 // The bit-packed target of a binary image: bit x % 32 of word x / 32 of row y
-// is pixel (x, y); rowpop [H + 1] the prefix sums of the rows' popcounts.
+// is pixel (x, y).
 struct DiscBits {
     const uint32_t* bits;   // null: the target is not binary
-    const int* rowpop;
+    const uint16_t* pre;    // [H][W + 1] (disc scenes)
+    int ones;               // set pixels of the target
 };
 
 // clamp of a float index estimate to [lo, hi] (NaN to lo)
@@ -191,36 +198,59 @@ __device__ __forceinline__ void exact_span(const float* ctr, int N, float fN, fl
     e = first_in(ic, N, guess_index(__fmaf_rn(__fadd_rn(c, half), fN, -0.5f), 0, N), [&](int i) { return !in(i); });
 }
 
+// Rows [y0, y1) that the disc at (cx, cy) can cover (see above; NaN: none)
+__device__ __forceinline__ void disc_band(int H, float cy, float radius, int& y0, int& y1) {
+    const float fH = (float)H;
+    const float mg = 2.0f + (fabsf(cy) + radius) * fH * 0x1p-20f;   // rows of margin
+    y0 = clamp_col(floorf(__fmaf_rn(__fsub_rn(cy, radius), fH, -0.5f) - mg), 0, H);
+    y1 = max(y0, clamp_col(ceilf(__fmaf_rn(__fadd_rn(cy, radius), fH, -0.5f) + mg) + 1.0f, 0, H));
+}
+
+// Row y's part of the mismatch count: the length of its covered interval less
+// twice the target's ones inside.
+__device__ __forceinline__ int disc_row(const uint16_t* __restrict__ pre, int W, float fW, const float* px, float py,
+                                        int y, float cx, float cy, float r2) {
+    const float dy = __fsub_rn(py, cy);
+    const float dy2 = __fmul_rn(dy, dy);
+    if (!(dy2 < r2)) return 0;
+    auto in = [&](int x) {
+        const float dx = __fsub_rn(px[x], cx);
+        return __fmaf_rn(dx, dx, dy2) < r2;
+    };
+    const float half = sqrtf(__fsub_rn(r2, dy2));
+    int a = guess_index(__fmaf_rn(__fsub_rn(cx, half), fW, -0.5f), 0, W);
+    int e = guess_index(__fmaf_rn(__fadd_rn(cx, half), fW, -0.5f), 0, W);
+    // (the four tests' indices stay inside the table whatever the guesses)
+    const bool a_in = in(min(a, W - 1)), a_out = in(max(a - 1, 0));
+    const bool e_in = in(max(e - 1, 0)), e_out = in(min(e, W - 1));
+    const bool sure = a < e && a_in && (a == 0 || !a_out) && e_in && (e == W || !e_out);
+    if (!sure) exact_span(px, W, fW, cx, half, in, a, e);
+    const uint16_t* p = pre + (size_t)y * (W + 1);
+    return a < e ? (e - a) - 2 * ((int)__ldg(p + e) - (int)__ldg(p + a)) : 0;
+}
+
 // Mismatch count of the disc at (cx, cy) against a binary target, summed over
-// the warp (every lane returns it): the rows [y0, y1) of the widened band go
-// to lanes y0 + lane, y0 + lane + 32, ...; the others come from the prefix sums.
+// the warp (every lane returns it), lanes over the rows.
 __device__ __forceinline__ int disc_mismatch_warp(const DiscBits& tb, int W, int H, const float* px,
                                                   const float* py, float cx, float cy, float radius, float r2,
                                                   int lane) {
-    const int words = (W + 31) >> 5;
-    const float fW = (float)W;
-    const float fH = (float)H;
-    const float mg = 2.0f + (fabsf(cy) + radius) * fH * 0x1p-20f;   // rows of margin (NaN: no rows)
-    const int y0 = clamp_col(floorf(__fmaf_rn(__fsub_rn(cy, radius), fH, -0.5f) - mg), 0, H);
-    const int y1 = max(y0, clamp_col(ceilf(__fmaf_rn(__fadd_rn(cy, radius), fH, -0.5f) + mg) + 1.0f, 0, H));
-    int cnt = lane == 0 ? __ldg(tb.rowpop + H) - (__ldg(tb.rowpop + y1) - __ldg(tb.rowpop + y0)) : 0;
-    for (int y = y0 + lane; y < y1; y += 32) {
-        const float dy = __fsub_rn(py[y], cy);
-        const float dy2 = __fmul_rn(dy, dy);
-        int a = 0, e = 0;
-        if (dy2 < r2)
-            exact_span(px, W, fW, cx, sqrtf(__fsub_rn(r2, dy2)), [&](int x) {
-                const float dx = __fsub_rn(px[x], cx);
-                return __fmaf_rn(dx, dx, dy2) < r2;
-            }, a, e);
-        const uint32_t* row = tb.bits + (size_t)y * words;
-        for (int j = 0; j < words; ++j) {
-            const int lo = min(max(a - 32 * j, 0), 32), hi = min(max(e - 32 * j, 0), 32);
-            const uint32_t m = (uint32_t)(((1ull << hi) - 1ull) & ~((1ull << lo) - 1ull));
-            cnt += __popc(__ldg(row + j) ^ m);
-        }
-    }
+    int y0, y1;
+    disc_band(H, cy, radius, y0, y1);
+    int cnt = lane == 0 ? tb.ones : 0;
+    for (int y = y0 + lane; y < y1; y += 32) cnt += disc_row(tb.pre, W, (float)W, px, py[y], y, cx, cy, r2);
     return __reduce_add_sync(0xffffffffu, cnt);
+}
+
+// The same count by one lane, for callers with a render per lane.
+__device__ __forceinline__ int disc_mismatch_lane(const DiscBits& tb, int W, int H, const float* px, const float* py,
+                                                  float cx, float cy, float radius) {
+    const float r2 = __fmul_rn(radius, radius);
+    int y0, y1;
+    disc_band(H, cy, radius, y0, y1);
+    int cnt = tb.ones;
+#pragma unroll 2
+    for (int y = y0; y < y1; ++y) cnt += disc_row(tb.pre, W, (float)W, px, py[y], y, cx, cy, r2);
+    return cnt;
 }
 
 // Loss of the disc at centre (cx, cy) against the target, by one warp (all

@@ -157,7 +157,9 @@ struct DevScene {
     // disc
     float radius = 0.f;
     uint32_t* tbits = nullptr;    // [H][(W + 31) / 32] bit-packed target (bit set: pixel is 1)
-    int* trowpop = nullptr;       // [H + 1] prefix sums of the packed rows' popcounts
+    int tones = 0;                // set pixels of the packed target
+    uint16_t* tpre = nullptr;     // [H][W + 1] ones of the packed rows by column (disc)
+    float* centres = nullptr;     // [W + H] FP32 pixel centres of the columns, then of the rows (disc)
     int tbinary = 0;              // 1: every target pixel is 0 or 1 (the loss is a mismatch count)
     // revolve
     float* verts = nullptr;       // [nv][3]
@@ -212,7 +214,7 @@ void revolve_prepare(DevScene& sc, cudaStream_t s);   // normals, kernel attribu
 void revolve_tile_t2(DevScene& sc, cudaStream_t s);   // after the target exists
 cudaError_t ptbox_prepare();   // kernel attributes
 cudaError_t tris2d_prepare_target(DevScene& sc, cudaStream_t s);   // after the target exists: sc.target4
-// disc and squares scenes, after the target exists: sc.tbits, sc.trowpop and sc.tbinary
+// disc and squares scenes, after the target exists: sc.tbits, sc.tbinary, sc.tones and (disc) sc.tpre, sc.centres
 cudaError_t disc_prepare_target(DevScene& sc, cudaStream_t s);
 
 int num_sms();

@@ -30,6 +30,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <deque>
 #include <mutex>
@@ -55,7 +56,11 @@ constexpr int kQUnitBits = 24;       // unit ring entry = request << 24 | unit
 constexpr unsigned long long kQUnitMask = (1ull << kQUnitBits) - 1ull;
 constexpr int kQUnitRing = 1 << 20;  // unit ring entries
 constexpr int kQReplicas = 8;        // device copies of each descriptor (unit k reads copy k % 8)
-constexpr int kQBatch = 4;           // descriptors the dispatcher loads per pass
+// Descriptors the dispatcher loads per pass: their loads from host memory are in
+// flight together, so a pass costs one such latency and one fence.  2,048
+// requests of 3 x 64 perturbations, which the dispatcher bounds: 2,032 us with 4
+// (and a load of its own for each request's units), 1,538 with 8, 1,752 with 16.
+constexpr int kQBatch = 8;
 
 // The sampler's inputs of a request (the fields sample_leg reads).
 struct QSample {
@@ -204,6 +209,7 @@ __device__ int dispatch_loop(const QArgs& A, int lane) {
         }
         hs = __shfl_sync(0xffffffffu, hs, 0);
         stop = __shfl_sync(0xffffffffu, stop, 0);
+        __syncwarp();   // lane 0's acquire is before every lane's descriptor loads
         if (hs > seen) {
             // kQBatch descriptors per pass: their host-memory loads are in
             // flight together; each is stored as kQReplicas device copies on
@@ -212,25 +218,29 @@ __device__ int dispatch_loop(const QArgs& A, int lane) {
             for (unsigned long long r0 = seen; r0 < hs; r0 += kQBatch) {
                 const int cnt = (int)min((unsigned long long)kQBatch, hs - r0);
                 int4 v[kQBatch];
-                int un[kQBatch];
 #pragma unroll
                 for (int j = 0; j < kQBatch; ++j) {
                     if (j >= cnt) break;
                     const int slot = (int)((r0 + j) % (unsigned long long)A.cap);
-                    if (lane < kQInt4) v[j] = __ldcv(reinterpret_cast<const int4*>(A.h_ring + slot) + lane);
-                    un[j] = __ldcv(&A.h_ring[slot].units);
+                    if (lane < kQInt4) v[j] = __ldcg(reinterpret_cast<const int4*>(A.h_ring + slot) + lane);
                 }
 #pragma unroll
                 for (int j = 0; j < kQBatch; ++j) {
                     if (j >= cnt) break;
                     const unsigned long long r = r0 + j;
                     const int slot = (int)(r % (unsigned long long)A.cap);
+                    // the request's units, from the lane that loaded them
+                    constexpr int kAt = (int)offsetof(QReq, units);
+                    const int un = __shfl_sync(0xffffffffu, kAt % 16 == 0   ? v[j].x
+                                                            : kAt % 16 == 4 ? v[j].y
+                                                            : kAt % 16 == 8 ? v[j].z
+                                                                            : v[j].w, kAt / 16);
                     if (lane < kQInt4)
                         for (int c = 0; c < kQReplicas; ++c)
                             __stcg(reinterpret_cast<int4*>(A.d_ring + (size_t)slot * kQReplicas + c) + lane, v[j]);
-                    for (int k = lane; k < un[j]; k += 32)
+                    for (int k = lane; k < un; k += 32)
                         __stcg(A.unit_ring + ((U + (unsigned long long)k) % kQUnitRing), (r << kQUnitBits) | (unsigned)k);
-                    U += (unsigned long long)un[j];
+                    U += (unsigned long long)un;
                 }
                 // publish each pass, so that workers start on a long backlog
                 __threadfence();
@@ -353,8 +363,20 @@ __global__ void __launch_bounds__(32 * kQWarps, 3) queue_kernel(QArgs A) {
                 sample_leg(R.sa, R.groups[g], R.lobes, p - g * R.P, lane & 1);
             }
             __syncwarp();
-            // 2. render the unit's perturbations, one after another by the whole warp
+            // 2. render the unit's perturbations: discs against a binary target one
+            //    per lane (a row's instructions serve 32 renders), the others one
+            //    after another by the whole warp.  512 requests of 3 x 1,024: 996 us
+            //    one after another with four tests per span end, 846 now; the
+            //    FP64 rate of the draws (590 us at least) is what remains.
             const int rows = 2 * min(kQPairs, pairs - p0);
+            if (kKind == HR_SCENE_DISC2D && A.tb.bits) {
+                if (lane < rows) {
+                    const float* t = R.sa.tau + (size_t)(2 * p0 + lane) * 2;   // this lane's own draw
+                    const float cx = __fadd_rn(R.theta32[0], t[0]), cy = __fadd_rn(R.theta32[1], t[1]);
+                    R.loss[2 * p0 + lane] = __fdiv_rn(
+                        (float)disc_mismatch_lane(A.tb, A.W, A.H, s_px, s_py, cx, cy, A.radius), (float)(A.W * A.H));
+                }
+            } else
             for (int q = 0; q < rows; ++q) {
                 const int m = 2 * p0 + q;
                 const float* t = R.sa.tau + (size_t)m * R.n;
@@ -518,7 +540,7 @@ hr_status ensure_running(hr_queue_s* q) {
     a.H = sc.H;
     a.radius = sc.radius;
     a.target = sc.target;
-    a.tb = DiscBits{sc.tbinary ? sc.tbits : nullptr, sc.trowpop};
+    a.tb = DiscBits{sc.tbinary ? sc.tbits : nullptr, sc.tpre, sc.tones};
     a.budget = q->budget;
     a.safety = q->safety;
     if (q->scene->sc.kind == HR_SCENE_DISC2D) queue_kernel<HR_SCENE_DISC2D><<<q->grid, 32 * kQWarps, 0, q->kstream>>>(a);

@@ -3,8 +3,6 @@
 // ((x + 1/2)/W, (y + 1/2)/H) is inside when fma(dx, dx, dy*dy) < r*r in FP32,
 // value 1 inside, 0 outside.  With a 0/1 target every (v - t)^2 is 0 or 1 and
 // the FP32 sum is an exact integer count.
-#include <vector>
-
 #include "disc_device.cuh"
 #include "hr.h"
 #include "hr_device.cuh"
@@ -16,24 +14,21 @@ namespace {
 template <int kW>
 __global__ void __launch_bounds__(32 * kW) disc_loss_kernel(RenderBatch b, int W, int H, float radius,
                                                             const float* __restrict__ target,
-                                                            DiscBits tb) {
-    __shared__ float s_px[HR_MAX_IMAGE_SIDE], s_py[HR_MAX_IMAGE_SIDE];
-    centre_tables(s_px, s_py, W, H);
-    __syncthreads();
+                                                            const float* __restrict__ centres, DiscBits tb) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m = blockIdx.x * kW + warp;
     if (m >= b.M) return;
     const Pert pt = resolve(b, m);
     const float cx = __fadd_rn(pt.theta[0], pt.tau[0]);
     const float cy = __fadd_rn(pt.theta[1], pt.tau[1]);
-    const float loss = disc_loss_warp(target, tb, W, H, radius, s_px, s_py, cx, cy, lane);
+    const float loss = disc_loss_warp(target, tb, W, H, radius, centres, centres + W, cx, cy, lane);
     if (lane == 0) *pt.loss = loss;
 }
 
 // Bit-packed target rows (bit x % 32 of word x / 32 of row y: pixel (x, y) is
-// 1) and a flag raised by any pixel other than 0 or 1.
+// 1), found[0] raised by any pixel other than 0 or 1, found[1] counting the ones.
 __global__ void disc_bits_kernel(const float* __restrict__ target, int W, int H, int words, uint32_t* bits,
-                                 int* non_binary) {
+                                 int* found) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= words * H) return;
     const int y = i / words, j = i - y * words;
@@ -45,7 +40,25 @@ __global__ void disc_bits_kernel(const float* __restrict__ target, int W, int H,
         else if (t != 0.0f) bad = true;
     }
     bits[i] = b;
-    if (bad) atomicOr(non_binary, 1);
+    if (bad) atomicOr(found, 1);
+    if (b) atomicAdd(found + 1, __popc(b));
+}
+
+// Tables of a disc scene: the pixel centres (columns, then rows) and, a block
+// per row, the target's ones by column, pre[y][x] in the first x pixels of row y.
+__global__ void disc_tables_kernel(const uint32_t* __restrict__ bits, int W, int H, int words, uint16_t* pre,
+                                   float* centres) {
+    const int y = blockIdx.x;
+    const uint32_t* row = bits + (size_t)y * words;
+    for (int x = threadIdx.x; x <= W; x += blockDim.x) {
+        int c = 0;
+        for (int j = 0; j < (x >> 5); ++j) c += __popc(__ldg(row + j));
+        if (x & 31) c += __popc(__ldg(row + (x >> 5)) & ((1u << (x & 31)) - 1u));
+        pre[(size_t)y * (W + 1) + x] = (uint16_t)c;
+    }
+    if (y == 0)
+        for (int i = threadIdx.x; i < W; i += blockDim.x) centres[i] = __fdiv_rn(__fadd_rn((float)i, 0.5f), (float)W);
+    if (threadIdx.x == 0) centres[W + y] = __fdiv_rn(__fadd_rn((float)y, 0.5f), (float)H);
 }
 
 __global__ void disc_image_kernel(const float* params, int W, int H, float radius, float* img) {
@@ -97,7 +110,7 @@ __global__ void boxes_image_kernel(const float* params, int K, int W, int H, flo
 // Launch-shape variants (autotuner): 8, 4 or 16 warps per CTA; one warp
 // renders one perturbation in every shape, so the choice never changes a result.
 void launch_boxes_loss(const DevScene& sc, const RenderBatch& b, cudaStream_t s) {
-    const DiscBits tb{sc.tbinary ? sc.tbits : nullptr, sc.trowpop};
+    const DiscBits tb{sc.tbinary ? sc.tbits : nullptr, sc.tpre, sc.tones};
     switch (sc.render_variant) {
         case 1: boxes_loss_kernel<4><<<(b.M + 3) / 4, 128, 0, s>>>(b, sc.W, sc.H, sc.radius, sc.target, tb); break;
         case 2: boxes_loss_kernel<16><<<(b.M + 15) / 16, 512, 0, s>>>(b, sc.W, sc.H, sc.radius, sc.target, tb); break;
@@ -111,42 +124,37 @@ void launch_boxes_image(const DevScene& sc, const float* params, float* img, cud
 }
 
 void launch_disc_loss(const DevScene& sc, const RenderBatch& b, cudaStream_t s) {
-    const DiscBits tb{sc.tbinary ? sc.tbits : nullptr, sc.trowpop};
+    const DiscBits tb{sc.tbinary ? sc.tbits : nullptr, sc.tpre, sc.tones};
     switch (sc.render_variant) {
-        case 1: disc_loss_kernel<4><<<(b.M + 3) / 4, 128, 0, s>>>(b, sc.W, sc.H, sc.radius, sc.target, tb); break;
-        case 2: disc_loss_kernel<16><<<(b.M + 15) / 16, 512, 0, s>>>(b, sc.W, sc.H, sc.radius, sc.target, tb); break;
-        default: disc_loss_kernel<8><<<(b.M + 7) / 8, 256, 0, s>>>(b, sc.W, sc.H, sc.radius, sc.target, tb); break;
+        case 1: disc_loss_kernel<4><<<(b.M + 3) / 4, 128, 0, s>>>(b, sc.W, sc.H, sc.radius, sc.target, sc.centres, tb); break;
+        case 2: disc_loss_kernel<16><<<(b.M + 15) / 16, 512, 0, s>>>(b, sc.W, sc.H, sc.radius, sc.target, sc.centres, tb); break;
+        default: disc_loss_kernel<8><<<(b.M + 7) / 8, 256, 0, s>>>(b, sc.W, sc.H, sc.radius, sc.target, sc.centres, tb); break;
     }
 }
 
+// One allocation: packed bits | what the packing found | centres | ones by column.
 cudaError_t disc_prepare_target(DevScene& sc, cudaStream_t s) {
     const int words = (sc.W + 31) / 32;
-    int* d_flag = nullptr;
-    cudaError_t e = cudaMalloc((void**)&sc.tbits, sizeof(uint32_t) * words * sc.H);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&d_flag, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemsetAsync(d_flag, 0, sizeof(int), s);
-    if (e == cudaSuccess) {
-        disc_bits_kernel<<<(words * sc.H + 255) / 256, 256, 0, s>>>(sc.target, sc.W, sc.H, words, sc.tbits, d_flag);
-        e = cudaGetLastError();
-    }
-    int non_binary = 1;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&non_binary, d_flag, sizeof(int), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFree(d_flag);
-    // prefix sums of the rows' popcounts (rows the disc cannot reach differ
-    // from the target in exactly its set pixels)
-    std::vector<uint32_t> bits((size_t)words * sc.H);
-    std::vector<int> pop((size_t)sc.H + 1, 0);
+    const bool disc = sc.kind == HR_SCENE_DISC2D;
+    const size_t n_bits = (size_t)words * sc.H, n_centres = disc ? (size_t)sc.W + sc.H : 0;
+    const size_t n_pre = disc ? (size_t)sc.H * (sc.W + 1) : 0;
+    cudaError_t e = cudaMalloc((void**)&sc.tbits, 4 * (n_bits + 2 + n_centres) + 2 * n_pre);
+    if (e != cudaSuccess) return e;
+    int* d_found = reinterpret_cast<int*>(sc.tbits + n_bits);
+    e = cudaMemsetAsync(d_found, 0, 2 * sizeof(int), s);
     if (e == cudaSuccess)
-        e = cudaMemcpy(bits.data(), sc.tbits, sizeof(uint32_t) * bits.size(), cudaMemcpyDeviceToHost);
-    for (int y = 0; y < sc.H; ++y) {
-        int c = 0;
-        for (int j = 0; j < words; ++j) c += __builtin_popcount(bits[(size_t)y * words + j]);
-        pop[y + 1] = pop[y] + c;
+        disc_bits_kernel<<<(words * sc.H + 255) / 256, 256, 0, s>>>(sc.target, sc.W, sc.H, words, sc.tbits, d_found);
+    if (e == cudaSuccess && disc) {
+        sc.centres = reinterpret_cast<float*>(d_found + 2);
+        sc.tpre = reinterpret_cast<uint16_t*>(sc.centres + n_centres);
+        disc_tables_kernel<<<sc.H, 128, 0, s>>>(sc.tbits, sc.W, sc.H, words, sc.tpre, sc.centres);
     }
-    if (e == cudaSuccess) e = cudaMalloc((void**)&sc.trowpop, sizeof(int) * pop.size());
-    if (e == cudaSuccess) e = cudaMemcpy(sc.trowpop, pop.data(), sizeof(int) * pop.size(), cudaMemcpyHostToDevice);
-    sc.tbinary = e == cudaSuccess && non_binary == 0;
+    int found[2] = {1, 0};
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(found, d_found, sizeof(found), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    sc.tbinary = e == cudaSuccess && found[0] == 0;
+    sc.tones = found[1];
     return e;
 }
 

@@ -456,6 +456,10 @@ void launch_sample(const SampleArgs& a, int n_groups, int max_P, cudaStream_t s)
     const size_t per_pair = 2 * (size_t)a.n * (sizeof(double) + sizeof(float));
     int np = legs / 2;
     while (np > 1 && np * per_pair > 40 * 1024) np /= 2;
+    // launches bound by the FP64 rate: enough pairs that the Gaussian units fill
+    // their warps (one dim in two of 16 pairs leaves half a warp idle)
+    if (np == 16 && (a.n & 3) == 2 && (int64_t)n_groups * max_P >= 32 * 8 * num_sms() && 32 * per_pair <= 40 * 1024)
+        np = 32;
     // many dims: spread few pairs over the SMs
     while (np > 2 && a.n >= 16 && (int64_t)n_groups * ((max_P + np - 1) / np) < num_sms()) np /= 2;
     const int units = 2 * ((2 * np + 31) / 32) + (np * ((a.n + 1) / 2) + 31) / 32;
