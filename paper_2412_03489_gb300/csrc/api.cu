@@ -517,6 +517,8 @@ hr_status hr_create_scene(const hr_scene_desc* d, hr_scene* out) {
             if ((e = cudaMalloc(&sc.tnrm, sizeof(float) * 3 * sc.nt)) != cudaSuccess) return bail(e, "normals");
             if ((e = cudaMalloc(&sc.tile_t2, sizeof(float) * revolve_tiles(sc))) != cudaSuccess)
                 return bail(e, "tiles");
+            if ((e = cudaMalloc(&sc.rv_target, sizeof(float) * 3 * 8 * sc.rv_th * revolve_tiles(sc))) != cudaSuccess)
+                return bail(e, "target tiles");
             if ((e = cudaMalloc(&sc.rv_stats, 8 * sizeof(unsigned long long))) != cudaSuccess) return bail(e, "stats");
             if ((e = cudaMemset(sc.rv_stats, 0, 8 * sizeof(unsigned long long))) != cudaSuccess) return bail(e, "stats");
             revolve_prepare(sc, s->stream);
@@ -585,6 +587,7 @@ hr_status hr_destroy_scene(hr_scene s) {
     DevScene& sc = s->sc;
     if (s->stream) cudaStreamSynchronize(s->stream);
     cudaFree(sc.target); cudaFree(sc.verts); cudaFree(sc.tris); cudaFree(sc.tnrm); cudaFree(sc.tile_t2);
+    cudaFree(sc.rv_target);
     cudaFree(sc.raw); cudaFree(sc.pidx); cudaFree(sc.target4); cudaFree(sc.qA); cudaFree(sc.qb); cudaFree(sc.rv_stats);
     cudaFree(sc.pt_stats); cudaFree(sc.tbits);   // (holds the other target tables)
     s->ws.release_all();

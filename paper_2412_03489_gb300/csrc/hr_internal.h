@@ -165,7 +165,8 @@ struct DevScene {
     float* verts = nullptr;       // [nv][3]
     int32_t* tris = nullptr;      // [nt][3]
     float* tnrm = nullptr;        // [nt][3] unit model-space normals (FP32)
-    float* tile_t2 = nullptr;     // [tiles] sum of target^2 per 8x8 tile
+    float* tile_t2 = nullptr;     // [tiles] sum of target^2 per tile
+    float* rv_target = nullptr;   // [tiles][rows][2][4][3] the target in tile order
     int nv = 0, nt = 0;
     float albedo[3] = {0, 0, 0}, light[3] = {0, 0, 0};
     float eye_dist = 0.f, scale = 0.f;

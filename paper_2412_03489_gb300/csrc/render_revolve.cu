@@ -103,7 +103,7 @@ struct RvArgs {
     const float* verts;
     const int32_t* tris;
     const float* tnrm;
-    const float* target;
+    const float* target_tiles;   // [T][kTH][2][4][3]: a lane's four pixels together
     const float* tile_t2;
     int nv, nt, W, H, TX, TY, T;
     int cap;             // bin entry capacity
@@ -208,7 +208,10 @@ __device__ int bin_scan(const int* cnt, OffT* off, uint16_t* olist, int T, int* 
 // E_i = fma(A_i, fx_c, r_i) > th_i for the three edges; it takes the entry
 // when also wz = fma(Aw, fx_c, rw) > bw_c (strict).  t4 becomes non-zero when
 // some wz == bw_c (an exact depth tie, resolved by a second, exact walk of
-// the tile).
+// the tile).  The raster is bound by instruction issue (about 73 a step, half of
+// the instructions of a 256x256 render): one LOP3 with a predicate result per pixel
+// for the two outside bits, in place of a LOP3 and a compare (with the target in
+// tile order, below: 182.4 M to 174.0 M warp instructions for 4,096 such renders).
 __device__ __forceinline__ void pixels4(const float4& q0, const float4& q1, const float4& q2, float Aw, float r0,
                                         float r1, float r2, float rw, const float fx[4], uint32_t outside,
                                         uint32_t row_out, int s, float bw[4], int bs[4], uint32_t& t4) {
@@ -218,13 +221,12 @@ __device__ __forceinline__ void pixels4(const float4& q0, const float4& q1, cons
         ".reg .f32 e0, e1, e2, w;\n\t"
         "setp.ne.u32 q, 0, 0;\n\t"
 #define HR_PIXEL(C, FX, BW, BS)                                 \
-        "lop3.b32 m, %18, %19, " #C ", 0xE0;\n\t"              \
-        "setp.eq.u32 p, m, 0;\n\t"                             \
+        "lop3.or.b32 m|p, %18, %19, " #C ", 0xE0, 0;\n\t"      \
         "fma.rn.f32 e0, %9, " FX ", %13;\n\t"                  \
         "fma.rn.f32 e1, %10, " FX ", %14;\n\t"                 \
         "fma.rn.f32 e2, %11, " FX ", %15;\n\t"                 \
         "fma.rn.f32 w, %12, " FX ", %16;\n\t"                  \
-        "setp.gt.and.f32 p, e0, %21, p;\n\t"                   \
+        "setp.gt.and.f32 p, e0, %21, !p;\n\t"                  \
         "setp.gt.and.f32 p, e1, %22, p;\n\t"                   \
         "setp.gt.and.f32 p, e2, %23, p;\n\t"                   \
         "setp.eq.or.f32 q, w, " BW ", q;\n\t"                  \
@@ -709,7 +711,6 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
             const int n_iter = all_tiles ? Tb : n_obj;
             const int col_shift = 4 * hx;
             const uint32_t row_out = 1u << (8 + ry - col_shift);   // this lane's row bit after the shift
-            const bool vec_target = (P.W & 3) == 0;
             // each warp reserves its next tiles when it starts the current ones,
             // so the shared atomic's latency overlaps the tiles' work
             int t_next = 0;
@@ -820,11 +821,10 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
                 float sh[4];
     #pragma unroll
                 for (int c = 0; c < 4; ++c) sh[c] = bs[c] != INT_MAX ? tshade[bs[c]] : 0.0f;
-                const bool rowv = has_tile && y < P.H;
                 if (kImage) {
     #pragma unroll
                     for (int c = 0; c < 4; ++c)
-                        if (rowv && x0 + c < P.W) {
+                        if (has_tile && y < P.H && x0 + c < P.W) {
                             const size_t q = (size_t)y * P.W + x0 + c;
                             if (ids) {
                                 ids[q] = bs[c] != INT_MAX ? bs[c] : -1;
@@ -833,28 +833,18 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
                             }
                         }
                 } else {
-                    float tg[12];
-                    if (rowv && vec_target && x0 + 3 < P.W) {
-                        const float4* tp = reinterpret_cast<const float4*>(P.target + 3 * ((size_t)y * P.W + x0));
-                        const float4 a0 = tp[0], a1 = tp[1], a2 = tp[2];
-                        tg[0] = a0.x; tg[1] = a0.y; tg[2] = a0.z; tg[3] = a0.w;
-                        tg[4] = a1.x; tg[5] = a1.y; tg[6] = a1.z; tg[7] = a1.w;
-                        tg[8] = a2.x; tg[9] = a2.y; tg[10] = a2.z; tg[11] = a2.w;
-                    } else {
-    #pragma unroll
-                        for (int c = 0; c < 4; ++c)
-    #pragma unroll
-                            for (int ch = 0; ch < 3; ++ch)
-                                tg[3 * c + ch] = (rowv && x0 + c < P.W) ? P.target[3 * ((size_t)y * P.W + x0 + c) + ch] : 0.0f;
-                    }
+                    // the target in tile order, this lane's 4 pixels together (pixels
+                    // outside the image are 0 there and no triangle covers them: they add 0)
+                    const float4* tp = reinterpret_cast<const float4*>(P.target_tiles) + 3 * (t * kG + gl);
+                    const float4 a0 = __ldg(tp), a1 = __ldg(tp + 1), a2 = __ldg(tp + 2);
+                    const float tg[12] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w, a2.x, a2.y, a2.z, a2.w};
                     float acc = 0.0f;
-    #pragma unroll
-                    for (int c = 0; c < 4; ++c)
-                        if (rowv && x0 + c < P.W) {
-                            const float d0 = sh[c] * P.alb0 - tg[3 * c], d1 = sh[c] * P.alb1 - tg[3 * c + 1];
-                            const float d2 = sh[c] * P.alb2 - tg[3 * c + 2];
-                            acc += d0 * d0 + d1 * d1 + d2 * d2;
-                        }
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        const float d0 = sh[c] * P.alb0 - tg[3 * c], d1 = sh[c] * P.alb1 - tg[3 * c + 1];
+                        const float d2 = sh[c] * P.alb2 - tg[3 * c + 2];
+                        acc += d0 * d0 + d1 * d1 + d2 * d2;
+                    }
                     // sum over the group's kG lanes
     #pragma unroll
                     for (int o = kG / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
@@ -945,9 +935,25 @@ __global__ void tile_t2_kernel(const float* target, int W, int H, int TX, int TH
     out[t] = s;
 }
 
+// The target in tile order, laid out once per scene, so that a lane's loads need
+// neither bounds checks nor an address from (x, y) and a warp's are contiguous: a
+// tile's fixed work is a third of a 512x512 render's.  Together with the LOP3 above,
+// before -> after per estimate: 256x256, 4,096 renders 844 -> 793 us; 400x400, 512
+// renders 259 -> 220 us; 512x512, 256 renders 215 -> 189 us; 128x128 no change.
+// Lane l of a tile (row l / 2, columns 4 (l % 2) to
+// 4 (l % 2) + 3) has its 12 values together, 0 outside the image
+__global__ void target_tiles_kernel(const float* target, int W, int H, int TX, int TH, int n, float* out) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;   // (tile, lane, pixel)
+    if (i >= n) return;
+    const int lanes = 2 * TH, c = i & 3, l = (i >> 2) % lanes, t = (i >> 2) / lanes;
+    const int ty = t / TX, x = (t - ty * TX) * kTW + 4 * (l & 1) + c, y = ty * TH + (l >> 1);
+    const bool in = x < W && y < H;
+    for (int k = 0; k < 3; ++k) out[3 * (size_t)i + k] = in ? target[3 * ((size_t)y * W + x) + k] : 0.0f;
+}
+
 RvArgs make_args(const DevScene& sc, bool compact = false, bool redo = false) {
     RvArgs a;
-    a.verts = sc.verts; a.tris = sc.tris; a.tnrm = sc.tnrm; a.target = sc.target; a.tile_t2 = sc.tile_t2;
+    a.verts = sc.verts; a.tris = sc.tris; a.tnrm = sc.tnrm; a.target_tiles = sc.rv_target; a.tile_t2 = sc.tile_t2;
     a.nv = sc.nv; a.nt = sc.nt; a.W = sc.W; a.H = sc.H;
     a.th = sc.rv_th;
     a.TX = (sc.W + kTW - 1) / kTW; a.TY = (sc.H + sc.rv_th - 1) / sc.rv_th; a.T = a.TX * a.TY;
@@ -1069,6 +1075,8 @@ void revolve_prepare(DevScene& sc, cudaStream_t s) {
 
 void revolve_tile_t2(DevScene& sc, cudaStream_t s) {
     const int TX = (sc.W + kTW - 1) / kTW, TY = (sc.H + sc.rv_th - 1) / sc.rv_th;
+    const int n = TX * TY * kTW * sc.rv_th;
+    target_tiles_kernel<<<(n + 255) / 256, 256, 0, s>>>(sc.target, sc.W, sc.H, TX, sc.rv_th, n, sc.rv_target);
     tile_t2_kernel<<<(TX * TY + 127) / 128, 128, 0, s>>>(sc.target, sc.W, sc.H, TX, sc.rv_th, TX * TY, sc.tile_t2);
 }
 
