@@ -521,7 +521,7 @@ hr_status hr_create_scene(const hr_scene_desc* d, hr_scene* out) {
                 return bail(e, "target tiles");
             if ((e = cudaMalloc(&sc.rv_stats, 8 * sizeof(unsigned long long))) != cudaSuccess) return bail(e, "stats");
             if ((e = cudaMemset(sc.rv_stats, 0, 8 * sizeof(unsigned long long))) != cudaSuccess) return bail(e, "stats");
-            revolve_prepare(sc, s->stream);
+            revolve_prepare(sc, maxsm, s->stream);
             break;
         }
         case HR_SCENE_TRIS2D:

@@ -211,7 +211,7 @@ int render_variant_count(int kind);
 // not fit
 bool revolve_layout(DevScene& sc, int max_smem, int smem_per_sm);
 int revolve_tiles(const DevScene& sc);
-void revolve_prepare(DevScene& sc, cudaStream_t s);   // normals, kernel attributes
+void revolve_prepare(DevScene& sc, int max_smem, cudaStream_t s);   // normals, kernel attributes
 void revolve_tile_t2(DevScene& sc, cudaStream_t s);   // after the target exists
 cudaError_t ptbox_prepare();   // kernel attributes
 cudaError_t tris2d_prepare_target(DevScene& sc, cudaStream_t s);   // after the target exists: sc.target4

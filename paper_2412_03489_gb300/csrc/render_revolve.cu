@@ -1056,17 +1056,19 @@ bool revolve_layout(DevScene& sc, int max_smem, int smem_per_sm) {
     return true;
 }
 
-void revolve_prepare(DevScene& sc, cudaStream_t s) {
+// The launch limits belong to the kernels, not to a scene: every scene sets the
+// largest that a layout can ask for, so that a small one made later does not
+// take a larger one's launches away.
+void revolve_prepare(DevScene& sc, int max_smem, cudaStream_t s) {
     normals_kernel<<<(sc.nt + 255) / 256, 256, 0, s>>>(sc.verts, sc.tris, sc.nt, sc.tnrm);
-    const int bytes = (int)sc.rv_smem;
+    const int bytes = max_smem - kStaticSmem;
     cudaFuncSetAttribute(revolve_kernel<4, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     cudaFuncSetAttribute(revolve_kernel<4, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     cudaFuncSetAttribute(revolve_kernel<8, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     cudaFuncSetAttribute(revolve_kernel<8, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (sc.rv_csmem) {
-        const int cb = (int)sc.rv_csmem;
-        cudaFuncSetAttribute(revolve_kernel<4, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, cb);
-        cudaFuncSetAttribute(revolve_kernel<8, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, cb);
+        cudaFuncSetAttribute(revolve_kernel<4, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        cudaFuncSetAttribute(revolve_kernel<8, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         // all of the SM's unified memory as shared memory, so that two CTAs fit
         cudaFuncSetAttribute(revolve_kernel<4, false, true>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
         cudaFuncSetAttribute(revolve_kernel<8, false, true>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);

@@ -28,3 +28,19 @@ def test_losses(size):
     # nothing covers), then trees: under 230 units of 2^-24, and shades of a few
     # units each, twice in a square: 2e-5 in all
     np.testing.assert_allclose(d["losses"], want, rtol=2e-5)
+
+
+def test_a_smaller_scene_made_later_leaves_a_larger_one_its_launches():
+    """The kernels' shared-memory limits are the process's: a scene with a small
+    layout made after one with a large layout does not lower them."""
+    big, th = wl.revolve_scene(width=512, height=512), np.asarray(wl.revolve_scene()["theta_query"], np.float64)
+    mid = wl.revolve_scene(width=64, height=64)
+    scenes = [hr.Scene(sc) for sc in (big, mid)]
+    before = [S.estimate(hr.HR_HESSIAN, th, 0.1, 4, hr.HR_AGGREGATE, 3, 4) for S in scenes]
+    small = dict(mid, width=8, height=8)
+    small["vertices"], small["triangles"] = wl.sheets_mesh(layers=1, grid=1)
+    late = hr.Scene(small)
+    after = [S.estimate(hr.HR_HESSIAN, th, 0.1, 4, hr.HR_AGGREGATE, 3, 4) for S in scenes]
+    for S in scenes + [late]:
+        S.close()
+    assert all(np.array_equal(a, b) for a, b in zip(after, before))
