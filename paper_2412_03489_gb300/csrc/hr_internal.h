@@ -171,7 +171,7 @@ struct DevScene {
     float albedo[3] = {0, 0, 0}, light[3] = {0, 0, 0};
     float eye_dist = 0.f, scale = 0.f;
     size_t rv_smem = 0;           // dynamic shared memory of one render
-    int rv_cap = 0, rv_vreg = 0;  // bin entry capacity, vertex-region floats
+    int rv_vreg = 0;              // vertex-region floats
     int rv_th = 8;                // raster tile height (8 x rv_th pixel tiles)
     size_t rv_csmem = 0;          // compact layout (two renders per SM): shared memory, 0 = none
     int rv_ccap = 0, rv_cslots = 0;   // its bin entry capacity and survivor slots
@@ -205,8 +205,8 @@ struct DevScene {
 int render_variant_count(int kind);
 
 // shared-memory layout and tile height of one mesh render on a device with
-// max_smem bytes of opt-in shared memory per block (sets rv_smem, rv_cap,
-// rv_vreg, rv_th) and, where it fits, of the compact layout that puts two
+// max_smem bytes of opt-in shared memory per block (sets rv_smem, rv_vreg,
+// rv_th) and, where it fits, of the compact layout that puts two
 // renders on an SM (rv_csmem, rv_ccap, rv_cslots); false if the mesh does
 // not fit
 bool revolve_layout(DevScene& sc, int max_smem, int smem_per_sm);

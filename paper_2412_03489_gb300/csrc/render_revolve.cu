@@ -9,18 +9,18 @@
 //            barrier-bound set-up phases overlap the other's raster; a render
 //            with more survivors than slots or more bin entries than fit is
 //            handed over (its loss set to a marker NaN);
-//   full     records by triangle, one CTA of 1024 threads per SM, bins that do
-//            not fit rastered in bands; it renders the handed-over
-//            perturbations (a second launch that reads the loss words), every
-//            scene too large for the compact layout, and images.
+//   full     room for a record of every triangle, one CTA of 1024 threads per
+//            SM; the bin entries follow the records that the render has, and
+//            bins that still do not fit are rastered in bands; it renders the
+//            handed-over perturbations (a second launch that reads the loss
+//            words), every scene too large for the compact layout, and images.
 // Both take the same coverage and depth decisions:
 //   1. rotation R = Rx(p0) Ry(p1) from RN32 of FP64 cos / sin (for every
 //      perturbation after a CTA's first, computed during the previous raster);
 //   2. vertex transform and projection (FP32, fixed operation order);
 //   3. triangle setup: edge functions with their top-left thresholds, back-face
 //      cull, depth plane of 1/Z, pixel bounding box, flat Lambert shade; each
-//      record stays at its triangle's index (full) or takes the next slot
-//      (compact, where the record carries the triangle's index);
+//      survivor takes the next slot and its record carries its index;
 //   4. binning into 8x4 pixel tiles (8x8 where shared memory is short; count,
 //      scan, fill; all in shared memory), skipping tiles that a conservative
 //      edge test shows the triangle misses; each bin entry carries the
@@ -70,9 +70,8 @@ constexpr uint32_t kTakenLoss = 0x7FC07A4Eu;
 
 // One surviving triangle.  E > 0, or E == 0 on a top-left edge, is one
 // compare: E > th with th = 0 or th = -(smallest subnormal) (no float lies
-// strictly between the two).  The last word is the flat shade (full layout:
-// records by triangle) or the triangle's index (compact layout: records by
-// survivor slot, the index decides depth ties); the raster reads the shades
+// strictly between the two).  The last word is the triangle's index (records are
+// by survivor slot, the index decides depth ties); the raster reads the shades
 // from their own array.
 struct __align__(16) TriRec {
     float A0, B0, C0, th0;
@@ -81,12 +80,9 @@ struct __align__(16) TriRec {
     float Aw, Bw, Cw, shade;
 };
 
-// bin entry: triangle << 16 | (tile rows OUTSIDE the bounding box) << 8 |
+// A bin entry is slot << 16 | (tile rows OUTSIDE the bounding box) << 8 |
 // (tile columns outside it): a pixel of the tile lies in the box iff neither
-// its row bit nor its column bit is set, one AND per pixel
-__device__ __forceinline__ uint32_t entry_word(int tri, uint32_t rows, uint32_t cols) {
-    return ((uint32_t)tri << 16) | ((~rows & 0xFFu) << 8) | (~cols & 0xFFu);
-}
+// its row bit nor its column bit is set, one AND per pixel.
 // an entry no pixel is in (record 0, every row and column outside)
 constexpr uint32_t kSentinel = 0x0000FFFFu;
 // bits lo..hi (clamped to 0..7) of a byte
@@ -106,7 +102,8 @@ struct RvArgs {
     const float* target_tiles;   // [T][kTH][2][4][3]: a lane's four pixels together
     const float* tile_t2;
     int nv, nt, W, H, TX, TY, T;
-    int cap;             // bin entry capacity
+    int cap;             // compact layout: bin entry capacity
+    int bytes;           // full layout: dynamic shared memory
     int vreg;            // floats in the vertex region
     int th;              // tile height (the kernel's template argument)
     int slots;           // compact layout: survivor slots (records by slot)
@@ -124,28 +121,6 @@ __device__ __forceinline__ bool pixel_range(float mn, float mx, int N, int& lo, 
     return lo <= hi;
 }
 
-// Does any pixel centre of tile (tx, ty) inside the triangle's bounding box
-// pass all three edge tests?  Conservative: false only when, for some edge,
-// the edge function at the corner of the (tile ∩ box) rectangle where it is
-// largest lies below neg[i] = -1e-5 (|A| W + |B| H + |C|), minus 1e-5 times
-// a bound on its term magnitudes anywhere in the image; the FP32 errors of
-// the exact per-pixel test and of this test are below 3e-7 of that
-// magnitude, so no rejected tile holds a covered pixel.
-template <int kTH>
-__device__ __forceinline__ bool tile_hits(const float A[3], const float B[3], const float C[3], uint2 bb,
-                                          const float neg[3], int tx, int ty) {
-    const int x0 = max(tx * kTW, (int)(bb.x & 0xffffu)), x1 = min(tx * kTW + kTW - 1, (int)(bb.x >> 16));
-    const int y0 = max(ty * kTH, (int)(bb.y & 0xffffu)), y1 = min(ty * kTH + kTH - 1, (int)(bb.y >> 16));
-    const float fx0 = (float)x0 + 0.5f, fx1 = (float)x1 + 0.5f, fy0 = (float)y0 + 0.5f, fy1 = (float)y1 + 0.5f;
-    bool hit = true;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        const float x = A[i] > 0.0f ? fx1 : fx0, y = B[i] > 0.0f ? fy1 : fy0;
-        hit = hit && !(fmaf(A[i], x, fmaf(B[i], y, C[i])) < neg[i]);
-    }
-    return hit;
-}
-
 constexpr int kCountClasses = 32;   // tiles ordered by entry count, counts >= 31 share a class
 
 // Exclusive scan of cnt[0..T) into off[0..T) and, in the same barriers, the
@@ -153,11 +128,15 @@ constexpr int kCountClasses = 32;   // tiles ordered by entry count, counts >= 3
 // largest first (a counting sort over count classes; the order within a
 // class is arbitrary, which only affects which warp takes which tile).  The
 // raster fetches the tiles of a warp together, one per lane group, so groups
-// of nearly equal counts waste few iterations, and the long tiles go first.  hist
-// [kCountClasses] must be zero on entry.  Returns the total entry count (all
+// of nearly equal counts waste few iterations, and the long tiles go first.
+// hist and cursor [kCountClasses] must be zero on entry.  Every warp scans the
+// warps' totals and the classes' for itself, which costs less than the barrier
+// that a scan by one warp needs.  Where the entries fit (total <= cap) cnt then
+// holds the offsets too, the fill's cursors.  Returns the total entry count (all
 // threads) and sets n_obj.
 template <int kT, class OffT>
-__device__ int bin_scan(const int* cnt, OffT* off, uint16_t* olist, int T, int* warp_tot, int* hist, int* n_obj) {
+__device__ int bin_scan(int* cnt, OffT* off, uint16_t* olist, int T, int* warp_tot, int* hist, int* cursor, int cap,
+                        int* n_obj) {
     const int per = (T + kT - 1) / kT;
     const int b = threadIdx.x * per;
     int local = 0;
@@ -168,38 +147,35 @@ __device__ int bin_scan(const int* cnt, OffT* off, uint16_t* olist, int T, int* 
             if (c > 0) atomicAdd(&hist[kCountClasses - 1 - min(c, kCountClasses - 1)], 1);
         }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int incl = local;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-    }
-    if (lane == 31) warp_tot[warp] = incl;
-    __syncthreads();
-    if (warp < 2) {   // warp 0: offsets of the warps' tile ranges; warp 1: the count classes
-        int* arr = warp == 0 ? warp_tot : hist;
-        const int wv = (warp == 0 && lane >= kT / 32) ? 0 : arr[lane];
-        int wi = wv;
+    auto scan = [&](int v) {   // inclusive, over the warp
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, wi, o);
-            if (lane >= o) wi += v;
+            const int u = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += u;
         }
-        arr[lane] = wi - wv;
-        if (lane == 31) arr[32] = wi;
-    }
+        return v;
+    };
+    const int incl = scan(local);
+    if (lane == 31) warp_tot[warp] = incl;
     __syncthreads();
-    int run = warp_tot[warp] + incl - local;
-    for (int i = 0; i < per; ++i)
+    const int wv = lane < kT / 32 ? warp_tot[lane] : 0, hv = hist[lane];
+    const int wi = scan(wv), hi = scan(hv);
+    const int total = __shfl_sync(0xffffffffu, wi, 31), first = hi - hv;   // first: of this lane's class in olist
+    int run = __shfl_sync(0xffffffffu, wi - wv, warp) + incl - local;
+    for (int i = 0; i < per; ++i) {
+        const int c = b + i < T ? cnt[b + i] : 0;
+        const int cls = kCountClasses - 1 - min(c, kCountClasses - 1);
+        const int at = __shfl_sync(0xffffffffu, first, cls);
         if (b + i < T) {
-            const int c = cnt[b + i];
             off[b + i] = (OffT)run;
-            if (c > 0) olist[atomicAdd(&hist[kCountClasses - 1 - min(c, kCountClasses - 1)], 1)] = (uint16_t)(b + i);
-            run += c;
+            if (total <= cap) cnt[b + i] = run;
+            if (c > 0) olist[at + atomicAdd(&cursor[cls], 1)] = (uint16_t)(b + i);
         }
+        run += c;
+    }
+    *n_obj = __shfl_sync(0xffffffffu, hi, 31);
     __syncthreads();
-    *n_obj = hist[32];
-    return warp_tot[32];
+    return total;
 }
 
 // The four pixels of a lane against one bin entry, as PTX predicate chains.
@@ -211,7 +187,7 @@ __device__ int bin_scan(const int* cnt, OffT* off, uint16_t* olist, int T, int* 
 // the tile).  The raster is bound by instruction issue (about 73 a step, half of
 // the instructions of a 256x256 render): one LOP3 with a predicate result per pixel
 // for the two outside bits, in place of a LOP3 and a compare (with the target in
-// tile order, below: 182.4 M to 174.0 M warp instructions for 4,096 such renders).
+// tile order, below: 182.4 M to 174.0 M warp instructions for 1,216 such renders).
 __device__ __forceinline__ void pixels4(const float4& q0, const float4& q1, const float4& q2, float Aw, float r0,
                                         float r1, float r2, float rw, const float fx[4], uint32_t outside,
                                         uint32_t row_out, int s, float bw[4], int bs[4], uint32_t& t4) {
@@ -287,9 +263,24 @@ __device__ __forceinline__ bool setup_triangle(const RvArgs& P, int ia, int ib, 
 // that two CTAs of 512 threads share an SM and one's barrier-bound set-up
 // phases overlap the other's raster; a render that does not fit (more
 // survivors than slots, more bin entries than the entry array) writes
-// kRedoLoss instead of its loss.  Otherwise (full layout) records by
-// triangle, one 1024-thread CTA per SM, bins too large for the shared memory
+// kRedoLoss instead of its loss.  Otherwise (full layout) room for records of
+// all triangles, one 1024-thread CTA per SM, bins too large for the shared memory
 // rastered in bands; with P.redo only the kRedoLoss perturbations are rendered.
+//
+// What a render of the compact layout spends (cycles of its 102 k at 256x256, 56 k
+// at 128x128; two renders share the SM's issue slots): raster 50 % / 36 %, count 15
+// / 14, fill 13 / 13, set-up 8 / 14, the rest scans, loads and reduction.  Issue is
+// active 67 %, so what was taken out: five of thirteen barriers (the rotation's
+// matrix is formed ahead too, every warp scans the totals, the scan leaves the
+// fill's cursors; 128x128, 2,048 renders: 228 -> 218 us per estimate); loops over
+// rows within loops over columns in count and fill (256x256, 4,096: 787 -> 755; count
+// 20.4 k -> 15.2 k cycles).  Records by slot in the full layout too: its entries
+// start behind the ~1,100 survivors of 2,048 triangles, so a 512x512 render's 5,800
+// fit at once instead of in two bands (512x512, 256 renders: 178 -> 153 us).  Tried
+// without gain: packed FMAs (fma.rn.f32x2) for pairs of edges, 4 % slower;
+// selects as predicated multiplies, the same; lanes on far-apart triangles in
+// count and fill, 2 % slower; two renders per SM in strips of rows for 512x512, 8 %
+// slower.
 template <int kTH, bool kImage, bool kCompact>
 __global__ void __launch_bounds__(kCompact ? kCompactThreads : kThreads, kCompact ? 2 : 1)
 revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, float* __restrict__ img,
@@ -301,18 +292,19 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
     using OffT = typename std::conditional<kCompact, uint16_t, int>::type;   // bin offsets (< kEntryCapMax)
     extern __shared__ __align__(16) unsigned char smem[];
     const int nrec = kCompact ? P.slots : P.nt;
-    TriRec* rec = reinterpret_cast<TriRec*>(smem);      // [nrec] by triangle (full) or by slot (compact)
-    uint2* bbx = reinterpret_cast<uint2*>(rec + nrec);  // [nrec] pixel bounding boxes
+    TriRec* rec;          // [nrec] survivors, by slot
+    uint2* bbx;           // [nrec] pixel bounding boxes
     float* vx;            // projected vertices x, y, 1/Z [nv] each
     float* tshade;        // [nrec] flat shades
     int* tcnt;            // [T] bin counts, then fill cursors, then tile losses
     OffT* toff;           // [T] bin offsets
-    uint16_t* surv = nullptr;              // full: [nt] surviving triangles (any order)
     uint32_t* ent;                         // [cap] bin entries
     unsigned long long* tmask = nullptr;   // full: [nt] tile masks of the count pass, by survivor
     uint16_t* tm16 = nullptr;              // compact: [slots] tile masks of rectangles of <= 16 tiles
     uint16_t* olist;                       // [T] tiles with entries, ordered by entry count
     if constexpr (kCompact) {
+        rec = reinterpret_cast<TriRec*>(smem);
+        bbx = reinterpret_cast<uint2*>(rec + nrec);
         tshade = reinterpret_cast<float*>(bbx + nrec);
         tcnt = reinterpret_cast<int*>(tshade + nrec);
         toff = reinterpret_cast<OffT*>(tcnt + P.T);
@@ -321,12 +313,15 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
         ent = reinterpret_cast<uint32_t*>(tm16 + ((nrec + 1) & ~1));
         vx = reinterpret_cast<float*>(ent);   // the vertices are dead before the first entry is written
     } else {
+        // the records last: the entries follow the last survivor's
+        bbx = reinterpret_cast<uint2*>(smem);
         vx = reinterpret_cast<float*>(bbx + nrec);   // vertex region, P.vreg floats (8 B aligned)
         tshade = vx + P.vreg;
         tcnt = reinterpret_cast<int*>(tshade + nrec);
         toff = reinterpret_cast<OffT*>(tcnt + P.T);
-        surv = reinterpret_cast<uint16_t*>(toff + P.T);
-        ent = reinterpret_cast<uint32_t*>(surv + ((P.nt + 1) & ~1));
+        const size_t at = (size_t)(reinterpret_cast<unsigned char*>(toff + P.T) - smem);
+        rec = reinterpret_cast<TriRec*>(smem + ((at + 15) & ~size_t(15)));
+        ent = nullptr;
         // after the triangle setup the vertex region holds the count pass's
         // tile masks and the list of tiles with entries
         tmask = reinterpret_cast<unsigned long long*>(vx);
@@ -335,12 +330,10 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
     float* vy = vx + P.nv;
     float* viz = vy + P.nv;
 
-    __shared__ float s_cs[4], s_cs_next[4];
-    __shared__ float sR[9];
-    __shared__ float sL[3];
+    __shared__ float s_rot[2][12];   // rotation and light of this render and, ahead, of the next
     __shared__ int s_count;
-    __shared__ int s_wtot[33];
-    __shared__ int s_hist[33];
+    __shared__ int s_wtot[32];
+    __shared__ int s_hist[2 * kCountClasses];   // count classes: tiles, then cursors
     __shared__ float s_part[kW];
     __shared__ int s_tile;
     __shared__ int s_band[2];   // the current band's end row and whether it walks every triangle
@@ -375,7 +368,7 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
     // free ones among the last 2G, so that CTAs that drew cheaper renders
     // take over the last renders of the others.  Each perturbation is
     // claimed, and rendered, exactly once.
-    __shared__ int s_pref;   // the perturbation claimed ahead (its rotation in s_cs_next), M if none
+    __shared__ int s_pref;   // the perturbation claimed ahead (its rotation in s_rot), M if none
     auto claim = [&](int i) -> bool {
         unsigned int* w = reinterpret_cast<unsigned int*>(resolve(b, i).loss);
         return atomicCAS(w, kFreeLoss, kTakenLoss) == kFreeLoss;
@@ -407,7 +400,28 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
         __syncthreads();
         return s_next;
     };
-    bool have_cs = false;   // compact: s_cs_next holds this perturbation's rotation
+    bool have_cs = false;   // compact: s_rot holds this perturbation's rotation
+    // one warp: rotation Rx(p0) Ry(p1) of perturbation mm from RN32 of FP64 cos / sin,
+    // and the light in model space, R^T l (shading value only)
+    auto rotate = [&](int mm, float* out) {
+        float v = 0.0f;
+        if (lane < 4) {
+            const float p = kImage ? img_params[lane >> 1] : rotation_param(b, mm, lane >> 1);
+            const double a = (double)p;
+            v = (float)((lane & 1) ? sin(a) : cos(a));
+        }
+        const float ca = __shfl_sync(0xffffffffu, v, 0), sa = __shfl_sync(0xffffffffu, v, 1);
+        const float cb = __shfl_sync(0xffffffffu, v, 2), sb = __shfl_sync(0xffffffffu, v, 3);
+        if (lane == 0) {
+            const float R[9] = {cb, 0.0f, sb, __fmul_rn(sa, sb), ca, -__fmul_rn(sa, cb),
+                                -__fmul_rn(ca, sb), sa, __fmul_rn(ca, cb)};
+#pragma unroll
+            for (int i = 0; i < 9; ++i) out[i] = R[i];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) out[9 + i] = R[i] * P.l0 + R[3 + i] * P.l1 + R[6 + i] * P.l2;
+        }
+    };
+    int cur = 1;   // s_rot's part of this render
     auto first_m = [&]() -> int {
         if constexpr (kImage) {
             return 0;
@@ -434,15 +448,12 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
     };
     for (int m = first_m(); m < M; m = next_m(m)) {
         // ---- 1. parameters and rotation ----------------------------------
-        if (tid < 4) {   // ca, sa, cb, sb
-            if (kCompact ? !have_cs : (kImage || m == (int)blockIdx.x || P.redo)) {
-                const float p = kImage ? img_params[tid >> 1] : rotation_param(b, m, tid >> 1);
-                const double a = (double)p;
-                s_cs[tid] = (float)((tid & 1) ? sin(a) : cos(a));
-            } else {
-                s_cs[tid] = s_cs_next[tid];   // computed during the previous raster phase
-            }
-        }
+        // (computed during the previous raster phase where there was one)
+        cur ^= 1;
+        const float* sR = s_rot[cur];
+        const float* sL = s_rot[cur] + 9;
+        const bool rotated = kCompact ? have_cs : !(kImage || m == (int)blockIdx.x || P.redo);
+        if (!rotated && warp == 0) rotate(m, s_rot[cur]);
         // scene constants this thread uses in the render (two vertices, two
         // triangles, the target's sum of squares on two tiles), loaded now so
         // that their latency overlaps the rotation
@@ -460,20 +471,9 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
             pt2[k] = (!kImage && tid + k * kT < P.T) ? P.tile_t2[tid + k * kT] : 0.0f;
         }
         for (int i = tid; i < P.T; i += kT) tcnt[i] = 0;
-        if (tid < 33) s_hist[tid] = 0;
+        if (tid < 2 * kCountClasses) s_hist[tid] = 0;
         if (tid == 0) { s_count = 0; s_tile = 0; }
-        __syncthreads();
-        if (tid == 0) {
-            const float ca = s_cs[0], sa = s_cs[1], cb = s_cs[2], sb = s_cs[3];
-            sR[0] = cb;                 sR[1] = 0.0f; sR[2] = sb;
-            sR[3] = __fmul_rn(sa, sb);  sR[4] = ca;   sR[5] = -__fmul_rn(sa, cb);
-            sR[6] = -__fmul_rn(ca, sb); sR[7] = sa;   sR[8] = __fmul_rn(ca, cb);
-            // light in model space: R^T l (shading value only)
-            sL[0] = sR[0] * P.l0 + sR[3] * P.l1 + sR[6] * P.l2;
-            sL[1] = sR[1] * P.l0 + sR[4] * P.l1 + sR[7] * P.l2;
-            sL[2] = sR[2] * P.l0 + sR[5] * P.l1 + sR[8] * P.l2;
-        }
-        __syncthreads();
+        if (!rotated) __syncthreads();
         // ---- 2. vertices ---------------------------------------------------
         const float halfW = __fmul_rn((float)P.W, 0.5f), halfH = __fmul_rn((float)P.H, 0.5f);
         auto project = [&](int v, float x, float y, float z) {
@@ -493,34 +493,20 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
             project(v, P.verts[3 * v], P.verts[3 * v + 1], P.verts[3 * v + 2]);
         __syncthreads();
         // ---- 3. triangle setup ------------------------------------------------
-        // records stay at their triangle's index (bin entries carry it for the
-        // tie rule); the survivors are listed for the binning, and a clipped,
-        // culled or off-image triangle gets an empty bounding box (lo > hi),
-        // which the all-triangles fallback of the raster skips
-        // (compact layout: a survivor takes the next slot; past the last slot
-        // it is only counted, and the render is handed to the full layout)
+        // a survivor takes the next slot and its record carries its index for the
+        // tie rule (compact layout: past the last slot it is only counted, and
+        // the render is handed to the full layout)
         auto setup = [&](int t, const int id[3], const float n[3]) {
             TriRec r;
             uint2 bb;
-            if constexpr (kCompact) {
-                if (setup_triangle(P, id[0], id[1], id[2], n, vx, vy, viz, sL, r, bb)) {
-                    const int k = atomicAdd(&s_count, 1);
-                    if (k < nrec) {
-                        tshade[k] = r.shade;
-                        r.shade = __int_as_float(t);
-                        rec[k] = r;
-                        bbx[k] = bb;
-                    }
+            if (setup_triangle(P, id[0], id[1], id[2], n, vx, vy, viz, sL, r, bb)) {
+                const int k = atomicAdd(&s_count, 1);
+                if (!kCompact || k < nrec) {
+                    tshade[k] = r.shade;
+                    r.shade = __int_as_float(t);
+                    rec[k] = r;
+                    bbx[k] = bb;
                 }
-            } else {
-                if (setup_triangle(P, id[0], id[1], id[2], n, vx, vy, viz, sL, r, bb)) {
-                    rec[t] = r;
-                    tshade[t] = r.shade;
-                    surv[atomicAdd(&s_count, 1)] = (uint16_t)t;
-                } else {
-                    bb = make_uint2(1u, 1u);
-                }
-                bbx[t] = bb;
             }
         };
 #pragma unroll
@@ -533,6 +519,11 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
         }
         __syncthreads();
         const int count = s_count;
+        int cap = P.cap;   // entries that the shared memory holds
+        if constexpr (!kCompact) {
+            ent = reinterpret_cast<uint32_t*>(rec + count);
+            cap = (int)((smem + P.bytes - reinterpret_cast<unsigned char*>(ent)) / sizeof(uint32_t));
+        }
         // (one warp, before the raster) the CTA's next perturbation and the
         // FP64 cos / sin of its rotation, off the critical path: full layout
         // m + G; compact, the next of its own that it claims (s_pref)
@@ -546,10 +537,7 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
             } else {
                 mn = m + (int)gridDim.x;
             }
-            if (lane < 4 && mn < M) {
-                const double a = (double)rotation_param(b, mn, lane >> 1);
-                s_cs_next[lane] = (float)((lane & 1) ? sin(a) : cos(a));
-            }
+            if (mn < M) rotate(mn, s_rot[cur ^ 1]);
         };
         // A compact-layout render that does not fit writes kRedoLoss (the full
         // layout renders it again) and claims the CTA's next perturbation,
@@ -569,55 +557,77 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
             }
         }
         // ---- 4. binning -----------------------------------------------------
-        // count pass: each survivor's tiles that pass the conservative edge
-        // test go into a bit mask (row-major over its tile rectangle;
-        // rectangles of more than 64 tiles, 16 in the compact layout, skip the
-        // test), reused by the fill
+        // count pass: each survivor's tiles that pass the edge test go into a bit
+        // mask (row-major over its tile rectangle; rectangles of more than 64
+        // tiles, 16 in the compact layout, skip the test), reused by the fill.
+        // The test is conservative: a tile is left out only when, for some edge,
+        // the edge function at the corner of the (tile ∩ box) rectangle where it
+        // is largest lies below neg = -1e-5 (|A| W + |B| H + |C|), minus 1e-5
+        // times a bound on its term magnitudes anywhere in the image; the FP32
+        // errors of the per-pixel test and of this one are below 3e-7 of that
+        // magnitude, so no tile that is left out holds a covered pixel.  One loop
+        // over the rectangle that steps to the next row in place (a loop in a
+        // loop runs for the warp's most rows times its most columns), with the
+        // tile's left edge kept as a float.
         for (int k = tid; k < count; k += kT) {
-            const int s = kCompact ? k : (int)surv[k];
-            const uint2 bb = bbx[s];
-            const float4* rp = reinterpret_cast<const float4*>(&rec[s]);
-            const float4 q0 = rp[0], q1 = rp[1], q2 = rp[2];
-            const float A[3] = {q0.x, q1.x, q2.x}, B[3] = {q0.y, q1.y, q2.y}, C[3] = {q0.z, q1.z, q2.z};
-            const int tx0 = (int)(bb.x & 0xffffu) / kTW, tx1 = (int)(bb.x >> 16) / kTW;
-            const int ty0 = (int)(bb.y & 0xffffu) / kTH, ty1 = (int)(bb.y >> 16) / kTH;
-            const bool test = (tx1 - tx0 + 1) * (ty1 - ty0 + 1) <= (kCompact ? 16 : 64);
-            const float fW = (float)P.W, fH = (float)P.H;
-            float neg[3];
-#pragma unroll
-            for (int i = 0; i < 3; ++i) neg[i] = -1e-5f * fmaf(fabsf(A[i]), fW, fmaf(fabsf(B[i]), fH, fabsf(C[i])));
-            unsigned long long mask = 0ull;
-            int bit = 0;
+            const uint2 bb = bbx[k];
             const int xlo = (int)(bb.x & 0xffffu), xhi = (int)(bb.x >> 16);
             const int ylo = (int)(bb.y & 0xffffu), yhi = (int)(bb.y >> 16);
-            for (int ty = ty0; ty <= ty1; ++ty) {
-                // per edge, the row term at the (tile row ∩ box) edge where
-                // B y is largest: the tile test is fma(A, x*, rowterm)
-                const float fy0 = (float)max(ty * kTH, ylo) + 0.5f, fy1 = (float)min(ty * kTH + kTH - 1, yhi) + 0.5f;
-                float rt[3];
+            const int tx0 = xlo / kTW, ty0 = ylo / kTH, nx = xhi / kTW - tx0 + 1, ny = yhi / kTH - ty0 + 1;
+            const int rect = nx * ny;
+            if (rect > (kCompact ? 16 : 64)) {
+                for (int ty = ty0; ty < ty0 + ny; ++ty)
+                    for (int tx = tx0; tx < tx0 + nx; ++tx) atomicAdd(&tcnt[ty * P.TX + tx], 1);
+                if constexpr (!kCompact) tmask[k] = ~0ull;
+                continue;
+            }
+            const float4* rp = reinterpret_cast<const float4*>(&rec[k]);
+            const float4 q0 = rp[0], q1 = rp[1], q2 = rp[2];
+            const float A[3] = {q0.x, q1.x, q2.x}, B[3] = {q0.y, q1.y, q2.y}, C[3] = {q0.z, q1.z, q2.z};
+            const float fW = (float)P.W, fH = (float)P.H;
+            const float fxl = (float)xlo + 0.5f, fxh = (float)xhi + 0.5f, fyl = (float)ylo + 0.5f, fyh = (float)yhi + 0.5f;
+            float neg[3], rt[3];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) neg[i] = -1e-5f * fmaf(fabsf(A[i]), fW, fmaf(fabsf(B[i]), fH, fabsf(C[i])));
+            const float left0 = (float)(tx0 * kTW) + 0.5f, right = (float)((tx0 + nx) * kTW);
+            float left = left0, top = (float)(ty0 * kTH) + 0.5f;
+            // per edge, the row term at the (tile row ∩ box) edge where B y is
+            // largest: the tile test is fma(A, x*, rowterm)
+            auto row_terms = [&]() {
+                const float fy0 = fmaxf(top, fyl), fy1 = fminf(top + (float)(kTH - 1), fyh);
 #pragma unroll
                 for (int i = 0; i < 3; ++i) rt[i] = fmaf(B[i], B[i] > 0.0f ? fy1 : fy0, C[i]);
-                for (int tx = tx0; tx <= tx1; ++tx, ++bit) {
-                    bool hit = true;
-                    if (test) {
-                        const float fx0 = (float)max(tx * kTW, xlo) + 0.5f, fx1 = (float)min(tx * kTW + kTW - 1, xhi) + 0.5f;
+            };
+            row_terms();
+            using Mask = typename std::conditional<kCompact, uint32_t, unsigned long long>::type;
+            Mask mask = 0;
+            int* cell = &tcnt[ty0 * P.TX + tx0];
+            for (int bit = 0; bit < rect; ++bit) {
+                const float fx0 = fmaxf(left, fxl), fx1 = fminf(left + (float)(kTW - 1), fxh);
+                bool hit = true;
 #pragma unroll
-                        for (int i = 0; i < 3; ++i) hit = hit && !(fmaf(A[i], A[i] > 0.0f ? fx1 : fx0, rt[i]) < neg[i]);
-                    }
-                    if (hit) {
-                        atomicAdd(&tcnt[ty * P.TX + tx], 1);
-                        if (test) mask |= 1ull << bit;
-                    }
+                for (int i = 0; i < 3; ++i) hit = hit && !(fmaf(A[i], A[i] > 0.0f ? fx1 : fx0, rt[i]) < neg[i]);
+                if (hit) {
+                    atomicAdd(cell, 1);
+                    mask |= (Mask)1 << bit;
+                }
+                left += (float)kTW;
+                ++cell;
+                if (left > right) {
+                    left = left0;
+                    top += (float)kTH;
+                    cell += P.TX - nx;
+                    row_terms();
                 }
             }
             if constexpr (kCompact) tm16[k] = (uint16_t)mask;
-            else tmask[k] = test ? mask : ~0ull;
+            else tmask[k] = mask;
         }
         __syncthreads();
         int n_obj = 0;
-        const int total = bin_scan<kT>(tcnt, toff, olist, P.T, s_wtot, s_hist, &n_obj);
+        const int total = bin_scan<kT>(tcnt, toff, olist, P.T, s_wtot, s_hist, s_hist + kCountClasses, cap, &n_obj);
         if constexpr (kCompact) {
-            if (total > P.cap) {
+            if (total > cap) {
                 hand_over();
                 continue;
             }
@@ -628,8 +638,8 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
         // entry array.  A tile row whose entries alone exceed capb is a band of
         // its own whose tiles walk every triangle.  A band only decides which
         // tiles are rastered together: every pixel's decisions are the same.
-        const bool banded = !kCompact && total > P.cap;
-        const int capb = banded ? P.cap - P.TY : P.cap;
+        const bool banded = !kCompact && total > cap;
+        const int capb = banded ? cap - P.TY : cap;
         int* rowtot = reinterpret_cast<int*>(ent) + capb;
         if (banded) {
             for (int r = warp; r < P.TY; r += kW) {
@@ -650,9 +660,6 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
         // the bins fit (then every argument but the row count is a constant)
         auto band = [&](const int r0, const int r1, const int total_b, const bool walk_all) {
             const int tb = r0 * P.TX, Tb = (r1 - r0) * P.TX;   // the band's tiles [tb, tb + Tb)
-            for (int i = tid; i < Tb; i += kT) tcnt[tb + i] = 0;   // becomes the fill cursor
-            if (tid == 0) s_tile = 0;
-            __syncthreads();
             if (!walk_all) {
                 // tiles without entries keep the sum of target^2 as their loss
                 // (the raster writes the others)
@@ -666,25 +673,38 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
                 for (int i = tid + 2 * kT; i < Tb; i += kT)
                     if (empty(i)) tl[tb + i] = P.tile_t2[tb + i];
                 for (int k = tid; k < count; k += kT) {
-                    const int s = kCompact ? k : (int)surv[k];
-                    const uint2 bb = bbx[s];
+                    const uint2 bb = bbx[k];
                     const int xlo = (int)(bb.x & 0xffffu), xhi = (int)(bb.x >> 16);
                     const int ylo = (int)(bb.y & 0xffffu), yhi = (int)(bb.y >> 16);
                     const int tx0 = xlo / kTW, tx1 = xhi / kTW, ty0 = ylo / kTH, ty1 = yhi / kTH;
+                    const int nx = tx1 - tx0 + 1, rect = nx * (ty1 - ty0 + 1);
                     const int ya = max(ty0, r0), yb = min(ty1, r1 - 1);
                     if (ya > yb) continue;
-                    unsigned long long mask;   // ~0: every tile of the rectangle (not tested)
-                    if constexpr (kCompact) mask = (tx1 - tx0 + 1) * (ty1 - ty0 + 1) <= 16 ? tm16[k] : ~0ull;
-                    else mask = tmask[k];
-                    int bit = (ya - ty0) * (tx1 - tx0 + 1);   // row-major over the whole tile rectangle
-                    for (int ty = ya; ty <= yb; ++ty) {
-                        // rows of this tile inside the box (bits >= kTH are never tested)
-                        const uint32_t rows = span_bits(ylo - ty * kTH, yhi - ty * kTH);
-                        for (int tx = tx0; tx <= tx1; ++tx, ++bit) {
-                            if (mask != ~0ull && !((mask >> bit) & 1ull)) continue;
-                            const int tile = ty * P.TX + tx;
-                            const int pos = atomicAdd(&tcnt[tile], 1);
-                            ent[toff[tile] + pos] = entry_word(s, rows, span_bits(xlo - tx * kTW, xhi - tx * kTW));
+                    // columns of the first and rows outside the box in the last tiles, as bits
+                    const uint32_t out_l = ~(0xFFu << (xlo & 7)) & 0xFFu, out_r = (0xFEu << (xhi & 7)) & 0xFFu;
+                    auto put = [&](int ty, int tx) {
+                        const uint32_t cols = (tx == tx0 ? out_l : 0u) | (tx == tx1 ? out_r : 0u);
+                        const uint32_t rows = span_bits(ylo - ty * kTH, yhi - ty * kTH);   // bits >= kTH are never tested
+                        ent[atomicAdd(&tcnt[ty * P.TX + tx], 1)] = ((uint32_t)k << 16) | ((~rows & 0xFFu) << 8) | cols;
+                    };
+                    if (rect > (kCompact ? 16 : 64)) {
+                        for (int ty = ya; ty <= yb; ++ty)
+                            for (int tx = tx0; tx <= tx1; ++tx) put(ty, tx);
+                        continue;
+                    }
+                    // the mask's set bits, lowest first; row of bit b: b / nx (exact for b, nx <= 64)
+                    const uint32_t recip = (65536u + (uint32_t)nx - 1u) / (uint32_t)nx;
+                    if constexpr (kCompact) {
+                        for (uint32_t mask = tm16[k]; mask; mask &= mask - 1u) {
+                            const uint32_t bit = (uint32_t)__ffs((int)mask) - 1u, row = (bit * recip) >> 16;
+                            put(ty0 + (int)row, tx0 + (int)(bit - row * (uint32_t)nx));
+                        }
+                    } else {
+                        unsigned long long mask = tmask[k];
+                        for (; mask; mask &= mask - 1ull) {
+                            const uint32_t bit = (uint32_t)__ffsll((long long)mask) - 1u, row = (bit * recip) >> 16;
+                            const int ty = ty0 + (int)row;
+                            if (ty >= ya && ty <= yb) put(ty, tx0 + (int)(bit - row * (uint32_t)nx));
                         }
                     }
                 }
@@ -764,13 +784,9 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
                             const float wz = __fmaf_rn(q3.x, fx[c], rw);
                             const bool in = ((outside & (row_out | (1u << c))) == 0u) && (E0 > q0.w) &&
                                             (E1 > q1.w) && (E2 > q2.w);
-                            // equal depths: the lower triangle index (records by
-                            // slot carry it in their last word)
-                            bool lower;
-                            if constexpr (kCompact)
-                                lower = bs[c] == INT_MAX || __float_as_int(rec[s].shade) < __float_as_int(rec[bs[c]].shade);
-                            else
-                                lower = s < bs[c];
+                            // equal depths: the lower triangle index (the record's last word)
+                            const bool lower =
+                                bs[c] == INT_MAX || __float_as_int(rec[s].shade) < __float_as_int(rec[bs[c]].shade);
                             const bool better = in && (wz > bw[c] || (wz == bw[c] && lower));
                             bw[c] = better ? wz : bw[c];
                             bs[c] = better ? s : bs[c];
@@ -806,15 +822,14 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
                         }
                     }
                 } else if constexpr (!kCompact) {
-                    // every triangle in index order (culled ones have an empty
-                    // box), so the strict compare already keeps the lower index
-                    for (int s = 0; s < P.nt; ++s) {
+                    // every survivor, with the full rule (slots are in no order)
+                    for (int s = 0; s < count; ++s) {
                         const uint2 bb = bbx[s];
                         const int xlo = (int)(bb.x & 0xffffu), xhi = (int)(bb.x >> 16);
                         const int ylo = (int)(bb.y & 0xffffu), yhi = (int)(bb.y >> 16);
-                        if (has_tile && xlo <= xhi && y >= ylo && y <= yhi)
+                        if (has_tile && y >= ylo && y <= yhi)
                             raster_entry(s, ((~span_bits(xlo - tx * kTW, xhi - tx * kTW) & 0xFFu) >> col_shift) & 0xFu,
-                                         false);
+                                         true);
                     }
                 }
                 // (every group runs the shuffles below, a group without a tile too)
@@ -827,7 +842,7 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
                         if (has_tile && y < P.H && x0 + c < P.W) {
                             const size_t q = (size_t)y * P.W + x0 + c;
                             if (ids) {
-                                ids[q] = bs[c] != INT_MAX ? bs[c] : -1;
+                                ids[q] = bs[c] != INT_MAX ? __float_as_int(rec[bs[c]].shade) : -1;
                             } else {
                                 img[3 * q] = sh[c] * P.alb0; img[3 * q + 1] = sh[c] * P.alb1; img[3 * q + 2] = sh[c] * P.alb2;
                             }
@@ -863,15 +878,16 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
                     while (r < P.TY && sum + rowtot[r] <= capb) sum += rowtot[r++];
                     s_band[0] = r > r0 ? r : r0 + 1;
                     s_band[1] = r > r0 ? 0 : 1;
+                    s_tile = 0;
                 }
-                if (tid < 33) s_hist[tid] = 0;
+                if (tid < 2 * kCountClasses) s_hist[tid] = 0;
                 __syncthreads();
                 r1 = s_band[0];
                 const bool walk_all = s_band[1] != 0;
                 walked = walked || walk_all;
                 const int total_b = walk_all ? 0
                                              : bin_scan<kT>(tcnt + r0 * P.TX, toff + r0 * P.TX, olist, (r1 - r0) * P.TX,
-                                                        s_wtot, s_hist, &n_obj);
+                                                        s_wtot, s_hist, s_hist + kCountClasses, capb, &n_obj);
                 band(r0, r1, total_b, walk_all);
             }
         }
@@ -892,7 +908,9 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
                 if (lane == 0) *resolve(b, m).loss = v / (float)(P.W * P.H * 3);
             }
         }
-        __syncthreads();
+        // (no barrier: what the next render writes before its first one, counters,
+        // vertices and the rotation ahead, was last read before the one above)
+        if (kImage) __syncthreads();
     }
     // each warp's raster steps go to the diagnostics once per launch
     if (!kImage && lane == 0 && P.stats && steps) atomicAdd(&P.stats[5], steps);
@@ -961,7 +979,8 @@ RvArgs make_args(const DevScene& sc, bool compact = false, bool redo = false) {
     a.alb0 = sc.albedo[0]; a.alb1 = sc.albedo[1]; a.alb2 = sc.albedo[2];
     a.l0 = sc.light[0]; a.l1 = sc.light[1]; a.l2 = sc.light[2];
     a.eye_dist = sc.eye_dist; a.scale = sc.scale;
-    a.cap = compact ? sc.rv_ccap : sc.rv_cap;
+    a.cap = sc.rv_ccap;
+    a.bytes = (int)sc.rv_smem;
     a.vreg = sc.rv_vreg;
     a.slots = sc.rv_cslots;
     a.redo = redo ? 1 : 0;
@@ -1014,16 +1033,17 @@ bool layout_for(int nv, int nt, int W, int H, int th, int max_smem, size_t* byte
 
 }  // namespace
 
-// Shared-memory layout of one render: records (64 B) and bounding boxes (8 B)
-// by triangle, the vertex region (the projected vertices, later the 64-bit
-// tile masks and the list of tiles with entries), shades (4 B) by triangle,
-// tile counts and offsets, the survivor list (2 B per triangle), and the bin
-// entries in what remains of max_smem (at most kEntryCapMax).  8x4 tiles
-// when that leaves room for 8,192 entries, else 8x8 tiles; false when fewer
-// than kEntryCapMin entries fit either way.  The tile height is a function of
-// the scene's sizes only (both layouts use it), so each layout sums a render's
-// loss in one fixed order, and which layout renders a perturbation depends on
-// that render's own survivors and entries only: results are deterministic.
+// Shared-memory layout of one render: bounding boxes (8 B) for every triangle,
+// the vertex region (the projected vertices, later the 64-bit tile masks and
+// the list of tiles with entries), shades (4 B), tile counts and offsets,
+// room for a record (64 B) of every triangle, and behind the records that a
+// render has, its bin entries.  8x4 tiles when the memory behind records of
+// all triangles (and 2 B for each of them) holds 8,192 entries, else 8x8
+// tiles; false when it holds fewer than kEntryCapMin either way.  The tile
+// height is a function of the scene's sizes only (both layouts use it), so each
+// layout sums a render's loss in one fixed order, and which layout renders a
+// perturbation depends on that render's own survivors and entries only: results
+// are deterministic.
 //
 // The compact layout (two CTAs per SM, each with half of smem_per_sm less
 // the 1 KB the hardware reserves per CTA) serves the renders it fits, with
@@ -1039,7 +1059,6 @@ bool revolve_layout(DevScene& sc, int max_smem, int smem_per_sm) {
         return false;
     }
     sc.rv_smem = bytes;
-    sc.rv_cap = cap;
     sc.rv_vreg = vreg;
     size_t cbytes = 0;
     int ccap = 0, cslots = 0;
