@@ -24,10 +24,10 @@ struct DevBuf {
 };
 
 struct Workspace {
-    DevBuf theta32, v, tau, w, meta, loss, flat, scale, full, groups, render_img, render_params;
+    DevBuf theta32, v, tau, w, meta, loss, flat, scale, full, render_img, render_params;
     DevBuf gb_J, gb_vx, gb_y, gb_vy, gb_out, gb_tmp, gb_hj;
     void release_all() {
-        for (DevBuf* b : {&theta32, &v, &tau, &w, &meta, &loss, &flat, &scale, &full, &groups, &render_img,
+        for (DevBuf* b : {&theta32, &v, &tau, &w, &meta, &loss, &flat, &scale, &full, &render_img,
                           &render_params, &gb_J, &gb_vx, &gb_y, &gb_vy, &gb_out, &gb_tmp, &gb_hj})
             b->release();
     }
@@ -40,7 +40,6 @@ struct hr_scene_s {
     std::mutex mu;
     cudaStream_t stream = nullptr;
     hr::Workspace ws;
-    std::vector<hr::SampleGroup> host_groups;
     bool profile = false;
     bool profile_valid = false;
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};

@@ -3,6 +3,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "hr.h"
+
 namespace hr {
 
 // One sample group: P antithetic pairs drawn for one component choice
@@ -22,8 +24,47 @@ struct SampleGroup {
     int32_t pad;
 };
 
+// The groups of an estimate: group g draws M / 2 pairs for element g
+// (element-wise; an HVP's row g by row-mixture draws) or, one group, from the
+// mixture (aggregate) or the plain Gaussian.
+struct GroupRule {
+    int32_t M, n, quantity, strategy;
+    uint32_t sub, request;
+    __host__ __device__ SampleGroup group(int g) const {
+        SampleGroup G;
+        G.m0 = g * M;
+        G.P = M / 2;
+        G.lobe = quantity == HR_GRAD ? 0 : 1;
+        G.quantity = quantity;
+        G.sub = sub + (uint32_t)g;
+        G.request = request;
+        G.theta_row = 0;
+        G.pad = 0;
+        if (strategy == HR_AGGREGATE) {
+            G.comp_i = G.comp_j = -1;
+        } else if (strategy == HR_PLAIN) {
+            G.comp_i = G.comp_j = -3;
+        } else if (quantity == HR_GRAD) {
+            G.comp_i = G.comp_j = g;
+        } else if (quantity == HR_HVP) {
+            G.comp_i = g;
+            G.comp_j = -2;
+            G.quantity = 4;
+        } else {   // element g of the upper triangle: row r starts at r n - r (r - 1) / 2
+            const float b = (float)(2 * n + 1);
+            int r = (int)(0.5f * (b - sqrtf(b * b - 8.0f * (float)g)));
+            while (r * n - r * (r - 1) / 2 > g) --r;
+            while ((r + 1) * n - (r + 1) * r / 2 <= g) ++r;
+            G.comp_i = r;
+            G.comp_j = r + g - (r * n - r * (r - 1) / 2);
+        }
+        return G;
+    }
+};
+
 struct SampleArgs {
-    const SampleGroup* groups;
+    const SampleGroup* groups;   // null: by `rule`
+    GroupRule rule;
     int32_t n;
     int32_t E;            // weight row width (0 if no weights written)
     double sigma;
@@ -37,9 +78,6 @@ struct SampleArgs {
     const int32_t* step;  // optional device step index s: every group's sub += 64 s
     const double* sigma_row;  // optional [rows]: group sigma = sigma_row[theta_row] (Z's derived in-kernel)
     int32_t threads;          // threads per block: 16, 32 (0 = 32), 64 or 128; no effect on the results
-    // up to kInlineGroups groups passed by value (n_inline > 0: groups[] is not read)
-    int32_t n_inline;
-    SampleGroup inline_groups[4];
     // optional: the first block also writes theta in FP32 (RN) to theta_out[theta_n],
     // from theta_in (device, FP64) or, when theta_in is null, from theta_vals
     const double* theta_in;
@@ -47,7 +85,6 @@ struct SampleArgs {
     int32_t theta_n;
     float theta_vals[64];
 };
-constexpr int kInlineGroups = 4;
 
 void launch_sample(const SampleArgs& a, int n_groups, int max_P, cudaStream_t s);
 

@@ -49,43 +49,6 @@ hr_status scratch_base(unsigned char** out) {
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
-// The sample-group table, written on the device so that the call needs no
-// host staging: group g draws P pairs for element g (element-wise) or from
-// the mixture (aggregate).
-__global__ void fill_groups_kernel(SampleGroup* groups, int G, int n, int quantity, int strategy, int M,
-                                   uint32_t sub, uint32_t request) {
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= G) return;
-    SampleGroup gr;
-    gr.m0 = g * M;
-    gr.P = M / 2;
-    gr.lobe = quantity == HR_GRAD ? 0 : 1;
-    gr.quantity = quantity;
-    gr.sub = sub + (uint32_t)g;
-    gr.request = request;
-    gr.theta_row = 0;
-    gr.pad = 0;
-    if (strategy == HR_AGGREGATE) {
-        gr.comp_i = -1; gr.comp_j = -1;
-    } else if (strategy == HR_PLAIN) {
-        gr.comp_i = -3; gr.comp_j = -3;
-    } else if (quantity == HR_GRAD) {
-        gr.comp_i = g; gr.comp_j = g;
-    } else if (quantity == HR_HVP) {
-        gr.comp_i = g; gr.comp_j = -2; gr.quantity = 4;
-    } else {
-        int r = 0, rem = g;
-        while (rem >= n - r) { rem -= n - r; ++r; }
-        gr.comp_i = r; gr.comp_j = r + rem;
-    }
-    groups[g] = gr;
-}
-
-__global__ void theta_to_f32_kernel(const double* in, float* out, int n) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = __double2float_rn(in[i]);
-}
-
 }  // namespace
 }  // namespace hr
 
@@ -130,12 +93,11 @@ extern "C" hr_status hr_estimate_dev_noalloc(hr_scene s, int32_t quantity, const
     cudaStream_t stream = o->stream ? (cudaStream_t)o->stream : s->stream;
 
     float* theta32 = reinterpret_cast<float*>(base + off_theta);
-    SampleGroup* groups = reinterpret_cast<SampleGroup*>(base + off_groups);
-    theta_to_f32_kernel<<<(n + 127) / 128, 128, 0, stream>>>(d_theta, theta32, n);
-    fill_groups_kernel<<<(G + 127) / 128, 128, 0, stream>>>(groups, G, n, quantity, o->strategy, (int)M, o->sub,
-                                                            o->request_id);
     SampleArgs sa{};
-    sa.groups = groups;
+    sa.theta_out = theta32;
+    sa.theta_in = d_theta;
+    sa.theta_n = n;
+    sa.rule = {(int32_t)M, n, quantity, o->strategy, o->sub, o->request_id};
     sa.n = n;
     sa.E = E;
     sa.sigma = o->sigma;

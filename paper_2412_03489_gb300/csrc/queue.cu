@@ -624,28 +624,8 @@ hr_status queue_push(hr_queue_s* q, int32_t quantity, const double* h_theta, con
     R.sa.w = reinterpret_cast<float*>(base + up256(sizeof(float) * Mt * n));
     R.loss = reinterpret_cast<float*>(base + up256(sizeof(float) * Mt * n) + up256(sizeof(float) * Mt * E));
     R.lobes = make_lobes(o->sigma, Zg, Zd, Zg * Zg, n);
-    for (int g = 0; g < G; ++g) {
-        SampleGroup& gr = R.groups[g];
-        gr.m0 = (int32_t)(g * o->n_perturb);
-        gr.P = P;
-        gr.lobe = quantity == HR_GRAD ? 0 : 1;
-        gr.quantity = quantity;
-        gr.sub = o->sub + (uint32_t)g;
-        gr.request = o->request_id;
-        if (o->strategy == HR_AGGREGATE) {
-            gr.comp_i = -1; gr.comp_j = -1;
-        } else if (o->strategy == HR_PLAIN) {
-            gr.comp_i = -3; gr.comp_j = -3;
-        } else if (quantity == HR_GRAD) {
-            gr.comp_i = g; gr.comp_j = g;
-        } else if (quantity == HR_HVP) {
-            gr.comp_i = g; gr.comp_j = -2; gr.quantity = 4;   // row g of the HVP, row-mixture draws
-        } else {
-            int r = 0, rem = g;
-            while (rem >= n - r) { rem -= n - r; ++r; }
-            gr.comp_i = r; gr.comp_j = r + rem;
-        }
-    }
+    const GroupRule rule{(int32_t)o->n_perturb, n, quantity, o->strategy, o->sub, o->request_id};
+    for (int g = 0; g < G; ++g) R.groups[g] = rule.group(g);
     R.res = q->dv_res + (size_t)slot * kQMaxResult;
     R.flag = q->dv_flag + slot;
     R.done = q->done + slot;

@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(kSampleThreads) sample_kernel(SampleArgs a, Lo
     __shared__ float2 s_c[128];
     __shared__ double s_sum[3 * 128];
     __shared__ Lobes s_lobes;
-    const SampleGroup G = a.n_inline > 0 ? a.inline_groups[blockIdx.y] : a.groups[blockIdx.y];
+    const SampleGroup G = a.groups ? a.groups[blockIdx.y] : a.rule.group((int)blockIdx.y);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, T = blockDim.x, n = a.n;
     if (a.theta_out && blockIdx.x == 0 && blockIdx.y == 0) {
         for (int d = tid; d < a.theta_n; d += T)

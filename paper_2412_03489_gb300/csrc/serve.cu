@@ -53,7 +53,6 @@ struct SrvReq {
     size_t off = 0, bytes = 0;
     float* theta32 = nullptr;
     double* vdev = nullptr;
-    SampleGroup* groups = nullptr;
     float* tau = nullptr;
     float* w = nullptr;
     uint2* meta = nullptr;
@@ -189,7 +188,7 @@ bool hr_server_s::admit(SrvReq* r) {
     return true;
 }
 
-// Upload parameters and group table, then sample every perturbation.
+// Upload parameters, then sample every perturbation.
 void hr_server_s::setup(SrvReq* r) {
     r->t_admit = now_ms();
     if (r->req.quantity == HR_NEWTON_STEP) {
@@ -205,41 +204,20 @@ void hr_server_s::setup(SrvReq* r) {
     size_t o = 0;
     r->theta32 = reinterpret_cast<float*>(b + o); o += up(sizeof(float) * n);
     r->vdev = reinterpret_cast<double*>(b + o); o += up(sizeof(double) * n);
-    r->groups = reinterpret_cast<SampleGroup*>(b + o); o += up(sizeof(SampleGroup) * (size_t)r->G);
+    o += up(sizeof(SampleGroup) * (size_t)r->G);
     r->tau = reinterpret_cast<float*>(b + o); o += up(sizeof(float) * (size_t)r->Mt * n);
     r->w = reinterpret_cast<float*>(b + o); o += up(sizeof(float) * (size_t)r->Mt * r->E);
     r->meta = reinterpret_cast<uint2*>(b + o); o += up(sizeof(uint2) * (size_t)r->Mt);
     r->loss = reinterpret_cast<float*>(b + o); o += up(sizeof(float) * (size_t)r->Mt);
     r->flat = reinterpret_cast<double*>(b + o); o += up(sizeof(double) * r->E);
     r->full = reinterpret_cast<double*>(b + o);
-    // staging: theta32 | v | groups, laid out as in the arena
-    const size_t head = up(sizeof(float) * n) + up(sizeof(double) * n) + up(sizeof(SampleGroup) * (size_t)r->G);
+    // staging: theta32 | v, laid out as in the arena
+    const size_t head = up(sizeof(float) * n) + up(sizeof(double) * n);
     std::vector<unsigned char> stage(head, 0);
     float* t32 = reinterpret_cast<float*>(stage.data());
     for (int i = 0; i < n; ++i) t32[i] = (float)r->theta[i];
     if (!r->v.empty()) memcpy(stage.data() + up(sizeof(float) * n), r->v.data(), sizeof(double) * n);
-    SampleGroup* gs = reinterpret_cast<SampleGroup*>(stage.data() + up(sizeof(float) * n) + up(sizeof(double) * n));
     const hr_opts& o2 = r->req.opts;
-    for (int g = 0; g < r->G; ++g) {
-        SampleGroup& gr = gs[g];
-        gr.m0 = (int32_t)(g * r->M);
-        gr.P = r->P;
-        gr.lobe = r->req.quantity == HR_GRAD ? 0 : 1;
-        gr.quantity = r->req.quantity;
-        gr.sub = o2.sub + (uint32_t)g;
-        gr.request = o2.request_id;
-        gr.theta_row = 0;
-        gr.pad = 0;
-        if (o2.strategy == HR_AGGREGATE) { gr.comp_i = -1; gr.comp_j = -1; }
-        else if (o2.strategy == HR_PLAIN) { gr.comp_i = -3; gr.comp_j = -3; }
-        else if (r->req.quantity == HR_GRAD) { gr.comp_i = g; gr.comp_j = g; }
-        else if (r->req.quantity == HR_HVP) { gr.comp_i = g; gr.comp_j = -2; gr.quantity = 4; }
-        else {
-            int row = 0, rem = g;
-            while (rem >= n - row) { rem -= n - row; ++row; }
-            gr.comp_i = row; gr.comp_j = row + rem;
-        }
-    }
     Lane& L = lane(r->req.scene);
     cudaError_t e = cudaMemcpyAsync(b, stage.data(), head, cudaMemcpyHostToDevice, upload);
     cudaEvent_t up_ev = get_event();
@@ -247,7 +225,7 @@ void hr_server_s::setup(SrvReq* r) {
     if (e == cudaSuccess) e = cudaStreamWaitEvent(L.stream, up_ev, 0);
     if (e != cudaSuccess) { r->status = HR_ERR_CUDA; put_event(up_ev); return; }
     SampleArgs sa{};
-    sa.groups = r->groups;
+    sa.rule = {(int32_t)r->M, n, r->req.quantity, o2.strategy, o2.sub, o2.request_id};
     sa.n = n;
     sa.E = r->E;
     sa.sigma = o2.sigma;
