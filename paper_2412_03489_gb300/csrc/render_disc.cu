@@ -17,6 +17,8 @@ __global__ void __launch_bounds__(32 * kW) disc_loss_kernel(RenderBatch b, int W
                                                             const float* __restrict__ centres, DiscBits tb) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m = blockIdx.x * kW + warp;
+    let_next_start();
+    wait_for_previous();
     if (m >= b.M) return;
     const Pert pt = resolve(b, m);
     const float cx = __fadd_rn(pt.theta[0], pt.tau[0]);
@@ -86,8 +88,10 @@ __global__ void __launch_bounds__(32 * kW) boxes_loss_kernel(RenderBatch b, int 
     __shared__ float s_c[kW][kMaxBoxParams];
     __shared__ int s_sp[kW][kMaxBoxParams];
     __shared__ float s_px[HR_MAX_IMAGE_SIDE], s_py[HR_MAX_IMAGE_SIDE];
+    let_next_start();
     centre_tables(s_px, s_py, W, H);
     __syncthreads();
+    wait_for_previous();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m = blockIdx.x * kW + warp;
     if (m >= b.M) return;
@@ -112,9 +116,9 @@ __global__ void boxes_image_kernel(const float* params, int K, int W, int H, flo
 void launch_boxes_loss(const DevScene& sc, const RenderBatch& b, cudaStream_t s) {
     const DiscBits tb{sc.tbinary ? sc.tbits : nullptr, sc.tpre, sc.tones};
     switch (sc.render_variant) {
-        case 1: boxes_loss_kernel<4><<<(b.M + 3) / 4, 128, 0, s>>>(b, sc.W, sc.H, sc.radius, sc.target, tb); break;
-        case 2: boxes_loss_kernel<16><<<(b.M + 15) / 16, 512, 0, s>>>(b, sc.W, sc.H, sc.radius, sc.target, tb); break;
-        default: boxes_loss_kernel<8><<<(b.M + 7) / 8, 256, 0, s>>>(b, sc.W, sc.H, sc.radius, sc.target, tb); break;
+        case 1: launch_after(boxes_loss_kernel<4>, dim3((b.M + 3) / 4), dim3(128), 0, s, b, sc.W, sc.H, sc.radius, sc.target, tb); break;
+        case 2: launch_after(boxes_loss_kernel<16>, dim3((b.M + 15) / 16), dim3(512), 0, s, b, sc.W, sc.H, sc.radius, sc.target, tb); break;
+        default: launch_after(boxes_loss_kernel<8>, dim3((b.M + 7) / 8), dim3(256), 0, s, b, sc.W, sc.H, sc.radius, sc.target, tb); break;
     }
 }
 
@@ -126,9 +130,9 @@ void launch_boxes_image(const DevScene& sc, const float* params, float* img, cud
 void launch_disc_loss(const DevScene& sc, const RenderBatch& b, cudaStream_t s) {
     const DiscBits tb{sc.tbinary ? sc.tbits : nullptr, sc.tpre, sc.tones};
     switch (sc.render_variant) {
-        case 1: disc_loss_kernel<4><<<(b.M + 3) / 4, 128, 0, s>>>(b, sc.W, sc.H, sc.radius, sc.target, sc.centres, tb); break;
-        case 2: disc_loss_kernel<16><<<(b.M + 15) / 16, 512, 0, s>>>(b, sc.W, sc.H, sc.radius, sc.target, sc.centres, tb); break;
-        default: disc_loss_kernel<8><<<(b.M + 7) / 8, 256, 0, s>>>(b, sc.W, sc.H, sc.radius, sc.target, sc.centres, tb); break;
+        case 1: launch_after(disc_loss_kernel<4>, dim3((b.M + 3) / 4), dim3(128), 0, s, b, sc.W, sc.H, sc.radius, sc.target, sc.centres, tb); break;
+        case 2: launch_after(disc_loss_kernel<16>, dim3((b.M + 15) / 16), dim3(512), 0, s, b, sc.W, sc.H, sc.radius, sc.target, sc.centres, tb); break;
+        default: launch_after(disc_loss_kernel<8>, dim3((b.M + 7) / 8), dim3(256), 0, s, b, sc.W, sc.H, sc.radius, sc.target, sc.centres, tb); break;
     }
 }
 

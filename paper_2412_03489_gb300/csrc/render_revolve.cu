@@ -340,6 +340,7 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int M = kImage ? 1 : b.M;
+    if (!kImage) { let_next_start(); wait_for_previous(); }
     unsigned long long steps = 0ull;   // lane 0: this warp's raster steps (diagnostics)
     // Redo mode: the first of this CTA's perturbations m0, m0 + G, ... (G the
     // grid) whose loss is kRedoLoss, M if none; warp 0 reads 32 loss words at
@@ -919,6 +920,8 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
 // every loss word of the launch to kFreeLoss (before a compact-layout launch)
 __global__ void mark_free_kernel(RenderBatch b) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    let_next_start();
+    wait_for_previous();
     if (i < b.M) *reinterpret_cast<unsigned int*>(resolve(b, i).loss) = kFreeLoss;
 }
 
@@ -1108,27 +1111,24 @@ int revolve_tiles(const DevScene& sc) {
 // With a compact layout: the loss words marked free, the compact launch (two
 // CTAs per SM), then the full-layout launch in redo mode, which renders only
 // the perturbations the compact one handed over (its CTAs read M loss words
-// when there are none).
+// when there are none).  That one starts after the compact launch's end: its
+// CTAs, early, would hold SMs that other streams' kernels could use (48 mixed
+// requests on the server: 6.05 ms, 6.34 so).
 void launch_revolve_loss(const DevScene& sc, const RenderBatch& b, cudaStream_t s) {
     if (b.M <= 0) return;   // nothing to render (and no empty grid to launch)
     const int grid = b.M < num_sms() ? b.M : num_sms();
     const bool compact = sc.rv_csmem != 0;
     if (compact) {
-        mark_free_kernel<<<(b.M + 255) / 256, 256, 0, s>>>(b);
+        launch_after(mark_free_kernel, dim3((b.M + 255) / 256), dim3(256), 0, s, b);
         const int cgrid = b.M < 2 * num_sms() ? b.M : 2 * num_sms();
-        if (sc.rv_th == 4)
-            revolve_kernel<4, false, true><<<cgrid, kCompactThreads, sc.rv_csmem, s>>>(make_args(sc, true), b, nullptr,
-                                                                                        nullptr, nullptr);
-        else
-            revolve_kernel<8, false, true><<<cgrid, kCompactThreads, sc.rv_csmem, s>>>(make_args(sc, true), b, nullptr,
-                                                                                        nullptr, nullptr);
+            const RvArgs ca = make_args(sc, true);
+        auto kernel = sc.rv_th == 4 ? revolve_kernel<4, false, true> : revolve_kernel<8, false, true>;
+        launch_after(kernel, dim3(cgrid), dim3(kCompactThreads), sc.rv_csmem, s, ca, b, nullptr, nullptr, nullptr);
     }
-    if (sc.rv_th == 4)
-        revolve_kernel<4, false, false><<<grid, kThreads, sc.rv_smem, s>>>(make_args(sc, false, compact), b, nullptr,
-                                                                           nullptr, nullptr);
-    else
-        revolve_kernel<8, false, false><<<grid, kThreads, sc.rv_smem, s>>>(make_args(sc, false, compact), b, nullptr,
-                                                                           nullptr, nullptr);
+    const RvArgs a = make_args(sc, false, compact);
+    auto kernel = sc.rv_th == 4 ? revolve_kernel<4, false, false> : revolve_kernel<8, false, false>;
+    if (compact) kernel<<<grid, kThreads, sc.rv_smem, s>>>(a, b, nullptr, nullptr, nullptr);
+    else launch_after(kernel, dim3(grid), dim3(kThreads), sc.rv_smem, s, a, b, nullptr, nullptr, nullptr);
 }
 
 // one image at params: colours into img [H][W][3], or, with ids non-null,

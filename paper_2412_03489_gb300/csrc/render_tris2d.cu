@@ -168,6 +168,7 @@ tris2d_loss_kernel(RenderBatch b, const float* __restrict__ raw, const int32_t* 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int m0 = blockIdx.x * kR;
     const int n_here = min(kR, b.M - m0);
+    let_next_start();
 #pragma unroll 1
     for (int r = 0; r < n_here; ++r) {
         const Pert pt = resolve(b, m0 + r);
@@ -361,6 +362,8 @@ __global__ void tris2d_target_kernel(const float* __restrict__ target, int W, in
 
 template <int kR>
 void launch_loss(const DevScene& sc, const RenderBatch& b, cudaStream_t s) {
+    // (not launch_after: blocks placed while the sampler's hold parts of the SMs stay
+    // unevenly spread; 64x64 Hessian of 1,024 renders 91 us, 105 so)
     tris2d_loss_kernel<kR><<<(b.M + kR - 1) / kR, kThreads, loss_bytes(kR, sc.n_tris, sc.W), s>>>(
         b, sc.raw, sc.pidx, sc.n_tris, sc.W, sc.H, reinterpret_cast<const float4*>(sc.target4));
 }

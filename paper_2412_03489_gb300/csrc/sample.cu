@@ -128,12 +128,12 @@ __global__ void __launch_bounds__(kSampleThreads) sample_kernel(SampleArgs a, Lo
     __shared__ float2 s_c[128];
     __shared__ double s_sum[3 * 128];
     __shared__ Lobes s_lobes;
+    let_next_start();
+    // without these the draws depend on nothing that an earlier kernel writes: they
+    // overlap the end of the previous estimate, and only the stores wait for it
+    if (a.groups || a.v || a.step || a.sigma_row) wait_for_previous();
     const SampleGroup G = a.groups ? a.groups[blockIdx.y] : a.rule.group((int)blockIdx.y);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, T = blockDim.x, n = a.n;
-    if (a.theta_out && blockIdx.x == 0 && blockIdx.y == 0) {
-        for (int d = tid; d < a.theta_n; d += T)
-            a.theta_out[d] = a.theta_in ? __double2float_rn(a.theta_in[d]) : a.theta_vals[d];
-    }
     const int kb = blockIdx.x * np;
     if (kb >= G.P) return;
     const int pairs = min(np, G.P - kb), rows = 2 * pairs;
@@ -215,6 +215,11 @@ __global__ void __launch_bounds__(kSampleThreads) sample_kernel(SampleArgs a, Lo
         }
     }
     __syncthreads();
+    wait_for_previous();
+    if (a.theta_out && blockIdx.x == 0 && blockIdx.y == 0) {
+        for (int d = tid; d < a.theta_n; d += T)
+            a.theta_out[d] = a.theta_in ? __double2float_rn(a.theta_in[d]) : a.theta_vals[d];
+    }
     const int m0 = G.m0 + 2 * kb;
     float* tau = a.tau + (size_t)m0 * n;
     for (int x = tid; x < rows * n; x += T) {
@@ -318,13 +323,13 @@ constexpr int kChunks = 256;
 // Kahan sums of rows [m, end): x and, with kAbs, |x|; the loads of sixteen rows
 // go out before their sums, which stay in row order.
 template <bool kAbs>
-__device__ __forceinline__ void chunk_sums(const float* __restrict__ w, const float* __restrict__ loss, int E, int e,
-                                           int m, int end, Kahan& ks, Kahan& ka) {
+__device__ __forceinline__ void chunk_sums(const float* w, const float* loss, int E, int e, int m, int end,
+                                           Kahan& ks, Kahan& ka) {
     auto batch = [&](auto count) {
         constexpr int kN = decltype(count)::value;
         float x[kN];
 #pragma unroll
-        for (int u = 0; u < kN; ++u) x[u] = __fmul_rn(__ldg(w + (size_t)(m + u) * E + e), __ldg(loss + m + u));
+        for (int u = 0; u < kN; ++u) x[u] = __fmul_rn(w[(size_t)(m + u) * E + e], loss[m + u]);
 #pragma unroll
         for (int u = 0; u < kN; ++u) {
             ks.add(x[u]);
@@ -355,6 +360,8 @@ __global__ void __launch_bounds__(kChunks) finalize_kernel(FinalizeArgs a) {
     const int e = blockIdx.x * kEl + el;
     const int m0 = (a.elementwise ? e * a.pairs2 : 0) + (int)blockIdx.y * a.row_stride;
     const int cnt = a.pairs2;
+    let_next_start();
+    wait_for_previous();
     const int chunk = (cnt + kChunks - 1) / kChunks;
     double s[kJ], sb[kAbs ? kJ : 1];
     if constexpr (kStaged) {
@@ -369,7 +376,7 @@ __global__ void __launch_bounds__(kChunks) finalize_kernel(FinalizeArgs a) {
             for (int k = 0; k < kRows; ++k) {
                 const int q = threadIdx.x + kChunks * k, row = r0 + q % kRows, m = (q / kRows) * chunk + row;
                 const bool in = row < chunk && m < cnt;
-                x[k] = in ? __fmul_rn(__ldg(a.w + (size_t)(m0 + m) * a.E + e), __ldg(a.loss + m0 + m)) : 0.0f;
+                x[k] = in ? __fmul_rn(a.w[(size_t)(m0 + m) * a.E + e], a.loss[m0 + m]) : 0.0f;
             }
 #pragma unroll
             for (int k = 0; k < kRows; ++k) {
@@ -442,8 +449,8 @@ __global__ void __launch_bounds__(kChunks) finalize_kernel(FinalizeArgs a) {
 template <int kEl, bool kStaged>
 void launch_finalize_as(const FinalizeArgs& a, cudaStream_t s) {
     const dim3 grid((a.E + kEl - 1) / kEl, a.batches > 0 ? a.batches : 1);
-    if (a.out_scale) finalize_kernel<kEl, true, kStaged><<<grid, kChunks, 0, s>>>(a);
-    else finalize_kernel<kEl, false, kStaged><<<grid, kChunks, 0, s>>>(a);
+    if (a.out_scale) launch_after(finalize_kernel<kEl, true, kStaged>, grid, dim3(kChunks), 0, s, a);
+    else launch_after(finalize_kernel<kEl, false, kStaged>, grid, dim3(kChunks), 0, s, a);
 }
 
 }  // namespace
@@ -465,7 +472,7 @@ void launch_sample(const SampleArgs& a, int n_groups, int max_P, cudaStream_t s)
     const int units = 2 * ((2 * np + 31) / 32) + (np * ((a.n + 1) / 2) + 31) / 32;
     const int T = units <= 4 ? 128 : kSampleThreads;
     dim3 grid((max_P + np - 1) / np, n_groups);
-    sample_kernel<<<grid, T, np * per_pair, s>>>(a, make_lobes(a.sigma, a.Zg, a.Zd, a.Zo, a.n), np);
+    launch_after(sample_kernel, grid, dim3(T), np * per_pair, s, a, make_lobes(a.sigma, a.Zg, a.Zd, a.Zo, a.n), np);
 }
 
 // Eight elements per block read whole sectors but give each thread eight times
