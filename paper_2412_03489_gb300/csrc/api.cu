@@ -171,7 +171,8 @@ hr_status run_estimate(hr_scene_s* s, int quantity, const double* h_theta, const
     WS_TRY(ws.v.reserve(sizeof(double) * n));
     WS_TRY(ws.tau.reserve(sizeof(float) * Mt * n));
     WS_TRY(ws.w.reserve(sizeof(float) * Mt * E));
-    WS_TRY(ws.meta.reserve(sizeof(uint2) * Mt));
+    const bool path_keys = sc.kind == HR_SCENE_PTBOX;   // only paths draw by perturbation
+    if (path_keys) WS_TRY(ws.meta.reserve(sizeof(uint2) * Mt));
     WS_TRY(ws.loss.reserve(sizeof(float) * Mt));
     WS_TRY(ws.flat.reserve(sizeof(double) * E));
     WS_TRY(ws.scale.reserve(sizeof(double) * E));
@@ -213,7 +214,7 @@ hr_status run_estimate(hr_scene_s* s, int quantity, const double* h_theta, const
     sa.tau = (float*)ws.tau.ptr;
     sa.w = (float*)ws.w.ptr;
     sa.invS = nullptr;
-    sa.meta = (uint2*)ws.meta.ptr;
+    sa.meta = path_keys ? (uint2*)ws.meta.ptr : nullptr;
     sa.threads = s->sc.sample_threads;
     if (s->profile) cudaEventRecord(s->ev[0], stream);
     launch_sample(sa, G, P, stream);
@@ -222,7 +223,7 @@ hr_status run_estimate(hr_scene_s* s, int quantity, const double* h_theta, const
     RenderBatch rb{};
     rb.theta32 = theta32;
     rb.tau = (const float*)ws.tau.ptr;
-    rb.meta = (const uint2*)ws.meta.ptr;
+    rb.meta = sa.meta;
     rb.loss = (float*)ws.loss.ptr;
     rb.M = (int32_t)Mt;
     rb.n = n;
@@ -285,8 +286,10 @@ hr_status run_hvp_fd(hr_scene_s* s, const double* h_theta, const double* h_v, do
     const int P = (int)(M / 2);
     const int64_t Mt = (int64_t)G * M;
     cudaStream_t stream = o->stream ? (cudaStream_t)o->stream : s->stream;
+    const bool path_keys = sc.kind == HR_SCENE_PTBOX;
     if (ws.theta32.reserve(sizeof(float) * 2 * n) != cudaSuccess || ws.tau.reserve(sizeof(float) * Mt * n) != cudaSuccess ||
-        ws.w.reserve(sizeof(float) * Mt * E) != cudaSuccess || ws.meta.reserve(sizeof(uint2) * Mt) != cudaSuccess ||
+        ws.w.reserve(sizeof(float) * Mt * E) != cudaSuccess ||
+        (path_keys && ws.meta.reserve(sizeof(uint2) * Mt) != cudaSuccess) ||
         ws.loss.reserve(sizeof(float) * 2 * Mt) != cudaSuccess || ws.flat.reserve(sizeof(double) * 3 * E) != cudaSuccess)
         return fail(HR_ERR_OOM, "workspace");
     std::vector<float> t32(2 * n);
@@ -308,7 +311,7 @@ hr_status run_hvp_fd(hr_scene_s* s, const double* h_theta, const double* h_v, do
     sa.seed = o->seed;
     sa.tau = (float*)ws.tau.ptr;
     sa.w = (float*)ws.w.ptr;
-    sa.meta = (uint2*)ws.meta.ptr;
+    sa.meta = path_keys ? (uint2*)ws.meta.ptr : nullptr;
     sa.threads = s->sc.sample_threads;
     launch_sample(sa, G, P, stream);
     RenderBatch rb{};
@@ -320,7 +323,7 @@ hr_status run_hvp_fd(hr_scene_s* s, const double* h_theta, const double* h_v, do
         BatchRow& br = rb.rows[r];
         br.theta32 = (const float*)ws.theta32.ptr + r * n;
         br.tau = (const float*)ws.tau.ptr;
-        br.meta = (const uint2*)ws.meta.ptr;
+        br.meta = sa.meta;
         br.loss = (float*)ws.loss.ptr + r * Mt;
         br.seed = o->seed;
         br.request = o->request_id;
