@@ -25,6 +25,7 @@
 #include "hr_api_internal.h"
 #include "hr_device.cuh"
 #include "hr_internal.h"
+#include "hvp_device.cuh"
 
 namespace hr {
 namespace {
@@ -62,7 +63,7 @@ struct NcgArgs {
 
 __global__ void __launch_bounds__(kNcgThreads) ncg_kernel(NcgArgs a) {
     __shared__ double d[kMaxN], r[kMaxN], q[kMaxN], red[kNcgThreads / 32];
-    __shared__ double tp[kMaxHvp];
+    __shared__ HvpTile tile;
     const int b = blockIdx.x, n = a.n;
     const double* g = a.g + (size_t)b * n;
     double* gd_ = a.d + (size_t)b * n;
@@ -101,21 +102,9 @@ __global__ void __launch_bounds__(kNcgThreads) ncg_kernel(NcgArgs a) {
     // Hd = 1/Mh sum_m loss_m (tau_m (tau_m.d)/s^4 - d/s^2) n^2/S(tau_m) + lambda d
     const double s2 = sigma * sigma, is2 = 1.0 / s2, is4 = is2 * is2;   // reciprocals: FP64 division is slow here
     const int m0 = b * a.per_inst + a.Mg;
-    for (int k = threadIdx.x; k < a.Mh; k += blockDim.x) {
-        const float* t = a.tau + (size_t)(m0 + k) * n;
-        double s = 0.0;
-        for (int c = 0; c < n; ++c) s += (double)t[c] * d[c];
-        tp[k] = s;
-    }
-    __syncthreads();
+    hvp_product(tile, a.tau + (size_t)m0 * n, a.invS + m0, a.loss + m0, a.Mh, n, d, is2, is4, q, [] {});
     for (int c = threadIdx.x; c < n; c += blockDim.x) {
-        Kahan acc;
-        for (int k = 0; k < a.Mh; ++k) {
-            const int m = m0 + k;
-            const double w = ((double)a.tau[(size_t)m * n + c] * tp[k] * is4 - d[c] * is2) * (double)a.invS[m];
-            acc.add(__fmul_rn((float)w, a.loss[m]));
-        }
-        const double hv = ((double)acc.s - (double)acc.c) / (double)a.Mh;
+        const double hv = q[c];
         q[c] = hv + lam * d[c];
         a.tr_q[(size_t)b * n + c] = hv;
     }

@@ -21,6 +21,7 @@
 #include "hr_api_internal.h"
 #include "hr_device.cuh"
 #include "hr_internal.h"
+#include "hvp_device.cuh"
 
 namespace hr {
 namespace {
@@ -49,7 +50,8 @@ struct CgArgs {
 
 __global__ void __launch_bounds__(kCgThreads) cg_kernel(CgArgs a) {
     __shared__ double d[kMaxN], r[kMaxN], p[kMaxN], Hp[kMaxN], red[kCgThreads / 32];
-    __shared__ double tp[512];
+    __shared__ HvpTile tile;
+    __shared__ double s_pn, s_cap;
     const int b = blockIdx.x, n = a.n;
     const double s2 = a.sigma * a.sigma, is2 = 1.0 / s2, is4 = is2 * is2;   // reciprocals: FP64 division is slow here
     const double* g = a.g + (size_t)b * n;
@@ -62,24 +64,20 @@ __global__ void __launch_bounds__(kCgThreads) cg_kernel(CgArgs a) {
     for (int it = 0; it < a.K; ++it) {
         iters = it + 1;
         const int m0 = b * a.per_inst + a.Mg + it * a.Mh;
-        // tau_m . p for the product's perturbations (n_hvp <= 512)
-        for (int q = threadIdx.x; q < a.Mh; q += blockDim.x) {
-            const float* t = a.tau + (size_t)(m0 + q) * n;
-            double s = 0.0;
-            for (int j = 0; j < n; ++j) s += (double)t[j] * p[j];
-            tp[q] = s;
-        }
-        __syncthreads();
-        // HVP_k = 1/Mh sum_m loss_m w_mk, w_mk = (tau_mk (tau_m.p)/s^4 - p_k/s^2) n^2/S(tau_m)
+        hvp_product(tile, a.tau + (size_t)m0 * n, a.invS + m0, a.loss + m0, a.Mh, n, p, is2, is4, Hp,
+                    [&] {   // |p| and the step that the trust region allows, as block_dot forms the sum
+                        const int lane = threadIdx.x & 31;
+                        double v0 = 0.0, v1 = 0.0;
+                        if (lane < n) v0 += p[lane] * p[lane];
+                        if (lane + 32 < n) v1 += p[lane + 32] * p[lane + 32];
+                        const double l = sqrt(warp_sum_d(v0) + warp_sum_d(v1));
+                        if (lane == 0) {
+                            s_pn = l;
+                            s_cap = a.delta / l;
+                        }
+                    });
         for (int k = threadIdx.x; k < n; k += blockDim.x) {
-            Kahan acc;
-            for (int q = 0; q < a.Mh; ++q) {
-                const int m = m0 + q;
-                const double tq = tp[q];
-                const double w = ((double)a.tau[(size_t)m * n + k] * tq * is4 - p[k] * is2) * (double)a.invS[m];
-                acc.add(__fmul_rn((float)w, a.loss[m]));
-            }
-            const double hv = ((double)acc.s - (double)acc.c) / (double)a.Mh;
+            const double hv = Hp[k];
             Hp[k] = hv + lam * p[k];
             const size_t tr = ((size_t)b * a.K + it) * n + k;
             a.tr_p[tr] = p[k];
@@ -87,7 +85,7 @@ __global__ void __launch_bounds__(kCgThreads) cg_kernel(CgArgs a) {
         }
         __syncthreads();
         const double pHp = block_dot(p, Hp, n, red);
-        const double pn = sqrt(block_dot(p, p, n, red));
+        const double pn = s_pn;
         if (!(pHp > 0.0) || pn == 0.0) {
             if (it == 0 && pn > 0.0)
                 for (int i = threadIdx.x; i < n; i += blockDim.x) d[i] = p[i] * (a.delta / pn);
@@ -95,7 +93,7 @@ __global__ void __launch_bounds__(kCgThreads) cg_kernel(CgArgs a) {
             __syncthreads();
             break;
         }
-        const double alpha = fmin(rr / pHp, a.delta / pn);
+        const double alpha = fmin(rr / pHp, s_cap);
         for (int i = threadIdx.x; i < n; i += blockDim.x) { d[i] += alpha * p[i]; r[i] -= alpha * Hp[i]; }
         __syncthreads();
         const double rr_new = block_dot(r, r, n, red);
