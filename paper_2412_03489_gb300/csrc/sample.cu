@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(kSampleThreads) sample_kernel(SampleArgs a, Lo
             if (r < rows) {
                 const PairDraw D = s_draw[r >> 1];
                 if (D.i >= 0 && (G.lobe == 0 ? b == 0 : D.i != D.j)) {
-                    const double x = sigma * sqrt(-2.0 * log(u01d(b ? D.ub : D.ua)));
+                    const double x = sigma * sqrt(-2.0 * log_pos(u01d(b ? D.ub : D.ua)));
                     float* t0 = s_t + (r - b) * n;   // the + leg's row; the - leg's follows
                     if (G.lobe == 0) {
                         t0[D.i] = (float)x;
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(kSampleThreads) sample_kernel(SampleArgs a, Lo
                 const bool need0 = d != D.i && d != D.j, need1 = d + 1 < n && d + 1 != D.i && d + 1 != D.j;
                 if (need0 || need1) {
                     const u32x4 r = philox_seed(a.seed, (uint32_t)(kb + p), (uint32_t)(1 + d / 4), c2, G.request);
-                    const double R = sqrt(-2.0 * log(u01d((d & 2) ? r.z : r.x)));
+                    const double R = sqrt(-2.0 * log_pos(u01d((d & 2) ? r.z : r.x)));
                     const double ph = 2.0 * kPi * u01d((d & 2) ? r.w : r.y);
                     double sn, cs;
                     sincos(ph, &sn, &cs);

@@ -7,6 +7,7 @@
 
 #include "hr_device.cuh"
 #include "hr_internal.h"
+#include "log_device.cuh"
 
 namespace hr {
 namespace {
@@ -30,7 +31,7 @@ __device__ __forceinline__ double recip_nr2(double x) {
 // Root s > 0 of  log(s) - s + 1 + L = 0  for L >= 0, i.e. s e^{-s} = e^{-1-L}.
 // upper: the root s >= 1 (tails of the diagonal lobe, |t| > 1), else s <= 1.
 // Halley's method on the log form.  A dependent FP64 operation costs tens of
-// cycles on this GPU, an FP64 log thousands, so:
+// cycles on this GPU, an FP64 log a thousand, so:
 //   1. away from the branch point (u = sqrt(2L) > 0.05) the start comes from
 //      the same iteration in FP32, begun at the branch-point expansion
 //      s = 1 +- u + u^2/3 or at the asymptotics of each branch; near it
@@ -38,7 +39,7 @@ __device__ __forceinline__ double recip_nr2(double x) {
 //   2. the FP64 iteration takes one log, of the start s0, and evaluates
 //      log s = log s0 + log1p(d), d = (s - s0)/s0, by the series of log1p
 //      (|d| <= 1e-4 on this path: the start is within ~1e-5 of the root;
-//      otherwise it falls back to log(s)); its divisions are Newton-refined
+//      otherwise it takes the log of s); its divisions are Newton-refined
 //      reciprocals (a step needs ~1e-14 relative, not a rounded quotient);
 //   3. it stops by the cubic convergence of Halley's method: after a step of
 //      relative size D the error is about D^3 / (4 (1 - s)^2), below 1e-17
@@ -75,18 +76,18 @@ __device__ double lobe_root(double L, bool upper) {
         if (u < (upper ? 2.0 : 1.0)) {
             s0 = 1.0 + (upper ? u : -u) + u * u * (1.0 / 3.0);
         } else if (upper) {
-            s0 = (1.0 + L) + log(1.0 + L);
+            s0 = (1.0 + L) + log_pos(1.0 + L);
         } else {
             const double y = exp(-1.0 - L);
             s0 = y * (1.0 + y);
         }
     }
-    const double lg0 = log(s0);
+    const double lg0 = log_pos(s0);
     const double r0 = recip_nr(s0);
     double s = s0;
     for (int it = 0; it < 16; ++it) {
         const double d = (s - s0) * r0;
-        const double ls = fabs(d) <= 1e-4 ? lg0 + d * (1.0 - d * (0.5 - d * (1.0 / 3.0 - 0.25 * d))) : log(s);
+        const double ls = fabs(d) <= 1e-4 ? lg0 + d * (1.0 - d * (0.5 - d * (1.0 / 3.0 - 0.25 * d))) : log_pos(s);
         const double g = ls - s + 1.0 + L;
         const double om = 1.0 - s;
         // Halley: s - 2 g g' / (2 g'^2 - g g''), g' = (1 - s)/s, g'' = -1/s^2
@@ -113,7 +114,7 @@ __device__ __forceinline__ double neg_log16(double m) {
     const double y = -((1.0 - 4.0 * m) * (1.0 + 4.0 * m));
     const bool direct = x < 0.5;
     const double w = 1.0 + y;
-    const double lg = log(direct ? x : w);
+    const double lg = log_pos(direct ? x : w);
     if (direct) return -lg;
     return w == 1.0 ? -y : -(y * (lg * recip_nr2(w - 1.0)));
 }
@@ -349,7 +350,7 @@ __device__ __forceinline__ void sample_leg(const Args& a, const SampleGroup& G, 
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             if (!(need[2 * q] || need[2 * q + 1])) continue;
-            const double R = sqrt(-2.0 * log(u01d(words[2 * q])));
+            const double R = sqrt(-2.0 * log_pos(u01d(words[2 * q])));
             const double ph = 2.0 * kPi * u01d(words[2 * q + 1]);
             if (need[2 * q]) g[d + 2 * q] = sigma * (R * cos(ph));
             if (need[2 * q + 1]) g[d + 2 * q + 1] = sigma * (R * sin(ph));
@@ -368,7 +369,7 @@ __device__ __forceinline__ void sample_leg(const Args& a, const SampleGroup& G, 
     }
     double vi, vj;   // this leg's values in dims i and j
     if (G.lobe == 0) {
-        const double r = sigma * sqrt(-2.0 * log(ua));
+        const double r = sigma * sqrt(-2.0 * log_pos(ua));
         vi = leg ? -r : r;
         vj = vi;
     } else if (i == j) {
@@ -377,8 +378,8 @@ __device__ __forceinline__ void sample_leg(const Args& a, const SampleGroup& G, 
         vi = sigma * diag_inverse(c);
         vj = vi;
     } else {
-        const double ri = sigma * sqrt(-2.0 * log(ua));
-        const double rj = sigma * sqrt(-2.0 * log(ub));
+        const double ri = sigma * sqrt(-2.0 * log_pos(ua));
+        const double rj = sigma * sqrt(-2.0 * log_pos(ub));
         const double sg = (w0.w & 1u) ? -1.0 : 1.0;
         vi = sg * ri;
         vj = leg ? -sg * rj : sg * rj;
