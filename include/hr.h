@@ -600,8 +600,9 @@ hr_status hr_profile_last(hr_scene scene, float* ms3);
 
 /* ---------------------------------------------------------------------------
  * Autotuning of launch shapes.  Each scene kind has render+loss launch-shape
- * variants (path tracer: minimum resident CTAs per SM 4 / 3 / 2, i.e. register
- * caps, 0 choosing by the size of launches that do not fill the GPU; disc and squares: 8 / 4 / 16 warps per CTA, one warp per
+ * variants (path tracer, where one CTA renders one perturbation: resident
+ * CTAs per SM, i.e. register caps, by the launch's size, 3 or 2; disc and
+ * squares: 8 / 4 / 16 warps per CTA, one warp per
  * perturbation; mesh and 2D triangles: one shape) and the sampler runs with
  * 16, 32, 64 or 128 threads per block (16 spreads small requests over more
  * SMs; with 64 or 128, a block takes its aggregate Hessian pairs diagonal-lobe

@@ -780,8 +780,8 @@ __device__ void load_pair(const PtArgs& A, PairShared& S) {
 
 // kSplit: the CTAs of a cluster render one pair, each a round of kSlots x 256
 // pixels at a time; rank 0 adds up their pixels in order.
-template <int kMinBlocks, int kSlots, bool kSplit>
-__global__ void __launch_bounds__(kThreads, kMinBlocks) ptbox_pair_kernel(PtArgs A, RenderBatch b) {
+template <int kSlots, bool kSplit>
+__global__ void __launch_bounds__(kThreads, 4) ptbox_pair_kernel(PtArgs A, RenderBatch b) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
     PairShared& S = *reinterpret_cast<PairShared*>(s_dyn);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1069,7 +1069,7 @@ void launch_parts(const PtArgs& a, const RenderBatch& b, int parts, cudaStream_t
     c.stream = s;
     c.attrs = &at;
     c.numAttrs = 1;
-    cudaLaunchKernelEx(&c, ptbox_pair_kernel<4, kSlots, true>, a, b);
+    cudaLaunchKernelEx(&c, ptbox_pair_kernel<kSlots, true>, a, b);
 }
 
 // CTAs that share one pair of renders (1: none) and the pixels per lane of their
@@ -1100,7 +1100,9 @@ PairShape pair_shape(int npx, int pairs, int sms) {
     return p;
 }
 
-void launch_pairs(int variant, const PtArgs& a, const RenderBatch& b, const PairShape& p, cudaStream_t s) {
+// (four CTAs per SM for every scene: 8,192 renders of 128x128, 4 spp take 42 ms,
+// 50 with three; a tuner's probe of 2,048 is split over clusters and cannot tell)
+void launch_pairs(const PtArgs& a, const RenderBatch& b, const PairShape& p, cudaStream_t s) {
     const int pairs = b.M / 2;
     if (p.parts > 1) {
         if (p.slots == 4) launch_parts<4>(a, b, p.parts, s);
@@ -1108,11 +1110,7 @@ void launch_pairs(int variant, const PtArgs& a, const RenderBatch& b, const Pair
         else launch_parts<1>(a, b, p.parts, s);
         return;
     }
-    switch (variant) {
-        case 1: ptbox_pair_kernel<3, kWhole, false><<<pairs, kThreads, pair_smem<kWhole>(), s>>>(a, b); break;
-        case 2: ptbox_pair_kernel<2, kWhole, false><<<pairs, kThreads, pair_smem<kWhole>(), s>>>(a, b); break;
-        default: ptbox_pair_kernel<4, kWhole, false><<<pairs, kThreads, pair_smem<kWhole>(), s>>>(a, b); break;
-    }
+    ptbox_pair_kernel<kWhole, false><<<pairs, kThreads, pair_smem<kWhole>(), s>>>(a, b);
 }
 
 template <bool kCanon>
@@ -1124,7 +1122,7 @@ void launch_loss(const DevScene& sc, const RenderBatch& b, cudaStream_t s) {
     }
     const PairShape p = kCanon && in_pairs(b) ? pair_shape(sc.W * sc.H, b.M / 2, num_sms()) : PairShape{};
     if (p.parts > 0) {
-        launch_pairs(sc.render_variant, a, b, p, s);
+        launch_pairs(a, b, p, s);
         return;
     }
     // variant 0: as many resident CTAs per SM as the launch has, 2 to 4 (fewer
@@ -1141,10 +1139,10 @@ void launch_loss(const DevScene& sc, const RenderBatch& b, cudaStream_t s) {
 
 }  // namespace
 
-// Launch-shape variants (autotuner): the same 256-thread layout and
-// arithmetic, different register caps through the minimum number of resident
-// CTAs per SM (4 or by the launch's size, 3, 2), so the choice never changes a
-// result.  Scenes with the procedural box's quad layout use the
+// Launch-shape variants (autotuner) of the kernel of one render per CTA: the same
+// 256-thread layout and arithmetic, different register caps through the minimum
+// number of resident CTAs per SM (by the launch's size, 3, 2), so the choice
+// never changes a result.  Scenes with the procedural box's quad layout use the
 // compile-time-axis intersection, and the pair kernel where it is faster.
 void launch_ptbox_loss(const DevScene& sc, const RenderBatch& b, cudaStream_t s) {
     if (canonical_axes(sc)) launch_loss<true>(sc, b, s);
@@ -1152,12 +1150,8 @@ void launch_ptbox_loss(const DevScene& sc, const RenderBatch& b, cudaStream_t s)
 }
 
 cudaError_t ptbox_prepare() {
-    cudaError_t e = cudaSuccess;
-    for (auto k : {ptbox_pair_kernel<2, kWhole, false>, ptbox_pair_kernel<3, kWhole, false>,
-                   ptbox_pair_kernel<4, kWhole, false>})
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pair_smem<kWhole>());
-    return e;
+    return cudaFuncSetAttribute(ptbox_pair_kernel<kWhole, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)pair_smem<kWhole>());
 }
 
 // One thread per pixel over as many blocks as it takes (a 64x64 target of 16 samples

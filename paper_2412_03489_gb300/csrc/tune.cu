@@ -15,7 +15,7 @@ namespace hr {
 
 int render_variant_count(int kind) {
     switch (kind) {
-        case HR_SCENE_PTBOX: return 3;     // min resident CTAs per SM 4 / 3 / 2 (register caps 64 / 80 / 128)
+        case HR_SCENE_PTBOX: return 3;     // one render per CTA: resident CTAs per SM by the launch, 3, 2 (register caps 64 to 128)
         case HR_SCENE_DISC2D: return 3;    // 8 / 4 / 16 warps per CTA, one warp per perturbation
         case HR_SCENE_BOXES2D: return 3;
         default: return 1;                 // mesh and 2D triangles: one CTA shape
