@@ -465,13 +465,16 @@ hr_status hr_create_scene(const hr_scene_desc* d, hr_scene* out) {
             }
             if ((e = upload(&sc.verts, d->vertices, 3 * (size_t)sc.nv)) != cudaSuccess) return bail(e, "vertices");
             if ((e = upload(&sc.tris, d->triangles, 3 * (size_t)sc.nt)) != cudaSuccess) return bail(e, "triangles");
-            if ((e = cudaMalloc(&sc.tnrm, sizeof(float) * 3 * sc.nt)) != cudaSuccess) return bail(e, "normals");
-            if ((e = cudaMalloc(&sc.tile_t2, sizeof(float) * revolve_tiles(sc))) != cudaSuccess)
-                return bail(e, "tiles");
-            if ((e = cudaMalloc(&sc.rv_target, sizeof(float) * 3 * 8 * sc.rv_th * revolve_tiles(sc))) != cudaSuccess)
-                return bail(e, "target tiles");
-            if ((e = cudaMalloc(&sc.rv_stats, 8 * sizeof(unsigned long long))) != cudaSuccess) return bail(e, "stats");
-            if ((e = cudaMemset(sc.rv_stats, 0, 8 * sizeof(unsigned long long))) != cudaSuccess) return bail(e, "stats");
+            // one allocation: target in tile order | counters | sums by tile | normals
+            const size_t tiles = revolve_tiles(sc), n_target = 3 * 8 * (size_t)sc.rv_th * tiles;
+            const size_t n_stats = 8 * sizeof(unsigned long long) / sizeof(float);
+            if ((e = cudaMalloc(&sc.rv_target, sizeof(float) * (n_target + n_stats + tiles + 3 * (size_t)sc.nt))) != cudaSuccess)
+                return bail(e, "mesh tables");
+            sc.rv_stats = reinterpret_cast<unsigned long long*>(sc.rv_target + n_target);
+            sc.tile_t2 = sc.rv_target + n_target + n_stats;
+            sc.tnrm = sc.tile_t2 + tiles;
+            if ((e = cudaMemsetAsync(sc.rv_stats, 0, 8 * sizeof(unsigned long long), s->stream)) != cudaSuccess)
+                return bail(e, "stats");
             revolve_prepare(sc, maxsm, s->stream);
             break;
         }
@@ -537,9 +540,9 @@ hr_status hr_destroy_scene(hr_scene s) {
     if (!s) return HR_OK;
     DevScene& sc = s->sc;
     if (s->stream) cudaStreamSynchronize(s->stream);
-    cudaFree(sc.target); cudaFree(sc.verts); cudaFree(sc.tris); cudaFree(sc.tnrm); cudaFree(sc.tile_t2);
-    cudaFree(sc.rv_target);
-    cudaFree(sc.raw); cudaFree(sc.pidx); cudaFree(sc.target4); cudaFree(sc.qA); cudaFree(sc.qb); cudaFree(sc.rv_stats);
+    cudaFree(sc.target); cudaFree(sc.verts); cudaFree(sc.tris);
+    cudaFree(sc.rv_target);   // (holds the other mesh tables)
+    cudaFree(sc.raw); cudaFree(sc.pidx); cudaFree(sc.target4); cudaFree(sc.qA); cudaFree(sc.qb);
     cudaFree(sc.pt_stats); cudaFree(sc.tbits);   // (holds the other target tables)
     s->ws.release_all();
     for (cudaEvent_t& e : s->ev)

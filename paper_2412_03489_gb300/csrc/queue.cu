@@ -366,8 +366,9 @@ __global__ void __launch_bounds__(32 * kQWarps, 3) queue_kernel(QArgs A) {
             // 2. render the unit's perturbations: discs against a binary target one
             //    per lane (a row's instructions serve 32 renders), the others one
             //    after another by the whole warp.  512 requests of 3 x 1,024: 996 us
-            //    one after another with four tests per span end, 846 now; the
-            //    FP64 rate of the draws (590 us at least) is what remains.
+            //    one after another with four tests per span end, 846 this way (732 with
+            //    eight descriptors a dispatcher pass and log_pos); the draws' FP64
+            //    operations are most of what remains.
             const int rows = 2 * min(kQPairs, pairs - p0);
             if (kKind == HR_SCENE_DISC2D && A.tb.bits) {
                 if (lane < rows) {

@@ -118,9 +118,10 @@ __device__ __forceinline__ void hessian_weights(const float* s_t, const double* 
 //
 // Bound by FP64 latency where the launch is small, by the FP64 rate (2 lanes a
 // cycle and SM) for many dims.  Stage times between events in us, with one leg
-// per thread and now: 3 x 1,024 element-wise 2 x 2: 18.2, 15.6; 4,096 aggregate
-// 2 x 2: 24.6, 18.0; 55 x 64 element-wise 10 x 10: 30.3, 16.5; 1,024 aggregate
-// 64 x 64 (2,080 weights each): 671, 34; 16,384 aggregate HVPs of 64 dims: 169, 95.
+// per thread and this way (both with log(); log_pos takes one to three off): 3 x 1,024
+// element-wise 2 x 2: 18.2, 15.6; 4,096 aggregate 2 x 2: 24.6, 18.0; 55 x 64 element-wise
+// 10 x 10: 30.3, 16.5; 1,024 aggregate 64 x 64 (2,080 weights each): 671, 34; 16,384
+// aggregate HVPs of 64 dims: 169, 95.
 __global__ void __launch_bounds__(kSampleThreads) sample_kernel(SampleArgs a, Lobes host_lobes, int np) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
     __shared__ PairDraw s_draw[64];

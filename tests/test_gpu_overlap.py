@@ -68,3 +68,34 @@ def test_calls_in_a_row(name, entry):
     for got in (run(False), bare(1), bare(5)):
         assert all(np.array_equal(a, b) for a, b in zip(got, want))
     S.close()
+
+
+@pytest.mark.parametrize("name", ["disc", "tris", "mesh", "path-traced"])
+def test_captured_calls(name):
+    """The no-allocation entry captured three times in a row into a graph (its first kernel has
+    no kernel before it there) and replayed: the results of the calls made alone."""
+    sc = SCENES[name]()
+    S, n = hr.Scene(sc), sc["n_params"]
+    theta = torch.tensor(np.asarray(sc["theta_query"], np.float64), device="cuda")
+    outs = [torch.zeros((n, n), dtype=torch.float64, device="cuda") for _ in range(3)]
+
+    def calls(stream):
+        for k, out in enumerate(outs):
+            o = hr.make_opts(sc["sigma"], 34, hr.HR_AGGREGATE, 3 + k, k, stream=stream.cuda_stream)
+            hr.hr_estimate_dev_noalloc(S.handle, hr.HR_HESSIAN, theta.data_ptr(), None, o, out.data_ptr())
+
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        calls(side)
+    torch.cuda.synchronize()
+    want = [x.cpu().numpy().copy() for x in outs]
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):
+        calls(side)
+    for _ in range(3):
+        for x in outs:
+            x.zero_()
+        graph.replay()
+    torch.cuda.synchronize()
+    assert all(np.array_equal(x.cpu().numpy(), w) for x, w in zip(outs, want))
+    S.close()
