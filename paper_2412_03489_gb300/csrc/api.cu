@@ -446,7 +446,10 @@ hr_status hr_create_scene(const hr_scene_desc* d, hr_scene* out) {
     };
     if (e != cudaSuccess) { delete s; return fail(HR_ERR_CUDA, "stream: %s", cudaGetErrorString(e)); }
     const size_t npx = (size_t)sc.W * sc.H * C;
-    if ((e = cudaMalloc(&sc.target, sizeof(float) * npx)) != cudaSuccess) return bail(e, "target");
+    // (a mesh has its target in tile order only: two copies of 786 KB each at 256x256
+    // made the allocator map another block per scene, a third of its creation)
+    const bool mesh = d->kind == HR_SCENE_REVOLVE3D;
+    if (!mesh && (e = cudaMalloc(&sc.target, sizeof(float) * npx)) != cudaSuccess) return bail(e, "target");
     switch (d->kind) {
         case HR_SCENE_DISC2D: sc.radius = d->radius; break;
         case HR_SCENE_BOXES2D: sc.radius = d->radius; break;
@@ -511,6 +514,13 @@ hr_status hr_create_scene(const hr_scene_desc* d, hr_scene* out) {
     if (analytic) {
         // no target: the loss is f itself
         if ((e = cudaMemset(sc.target, 0, sizeof(float) * npx)) != cudaSuccess) return bail(e, "target");
+    } else if (d->target_image && mesh) {
+        float* image = nullptr;
+        if ((e = upload(&image, d->target_image, npx)) != cudaSuccess) return bail(e, "target upload");
+        revolve_tables(sc, image, s->stream);
+        e = cudaStreamSynchronize(s->stream);
+        cudaFree(image);
+        if (e != cudaSuccess) return bail(e, "target tiles");
     } else if (d->target_image) {
         if ((e = cudaMemcpy(sc.target, d->target_image, sizeof(float) * npx, cudaMemcpyHostToDevice)) != cudaSuccess)
             return bail(e, "target upload");
@@ -519,12 +529,16 @@ hr_status hr_create_scene(const hr_scene_desc* d, hr_scene* out) {
         for (int i = 0; i < sc.n; ++i) p32[i] = (float)d->theta_target[i];
         float* dp = nullptr;
         if ((e = upload(&dp, p32.data(), (size_t)sc.n)) != cudaSuccess) return bail(e, "target params");
-        launch_render_image(sc, dp, sc.scene_seed, 0, 0, 0, hr::TAG_TARGET, sc.target_spp, sc.target, s->stream);
+        if (mesh) {
+            launch_revolve_target(sc, dp, s->stream);
+            revolve_tables(sc, nullptr, s->stream);
+        } else {
+            launch_render_image(sc, dp, sc.scene_seed, 0, 0, 0, hr::TAG_TARGET, sc.target_spp, sc.target, s->stream);
+        }
         e = cudaStreamSynchronize(s->stream);
         cudaFree(dp);
         if (e != cudaSuccess) return bail(e, "target render");
     }
-    if (sc.kind == HR_SCENE_REVOLVE3D) revolve_tile_t2(sc, s->stream);
     if (sc.kind == HR_SCENE_TRIS2D && (e = tris2d_prepare_target(sc, s->stream)) != cudaSuccess)
         return bail(e, "target tiles");
     if ((sc.kind == HR_SCENE_DISC2D || sc.kind == HR_SCENE_BOXES2D) &&

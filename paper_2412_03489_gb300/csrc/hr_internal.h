@@ -249,7 +249,9 @@ int render_variant_count(int kind);
 bool revolve_layout(DevScene& sc, int max_smem, int smem_per_sm);
 int revolve_tiles(const DevScene& sc);
 void revolve_prepare(DevScene& sc, int max_smem, cudaStream_t s);   // normals, kernel attributes
-void revolve_tile_t2(DevScene& sc, cudaStream_t s);   // after the target exists
+void launch_revolve_target(const DevScene& sc, const float* params, cudaStream_t s);   // into rv_target
+// the sums by tile, and before them rv_target from an image [H][W][3] if one is given
+void revolve_tables(DevScene& sc, const float* image, cudaStream_t s);
 cudaError_t ptbox_prepare();   // kernel attributes
 cudaError_t tris2d_prepare_target(DevScene& sc, cudaStream_t s);   // after the target exists: sc.target4
 // disc and squares scenes, after the target exists: sc.tbits, sc.tbinary, sc.tones and (disc) sc.tpre, sc.centres

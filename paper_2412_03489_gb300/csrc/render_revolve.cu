@@ -107,6 +107,7 @@ struct RvArgs {
     int vreg;            // floats in the vertex region
     int th;              // tile height (the kernel's template argument)
     int slots;           // compact layout: survivor slots (records by slot)
+    int tiled;           // image: in the target's tile order, zeros outside
     int redo;            // full layout: render only the perturbations whose loss is kRedoLoss
     uint64_t tx_recip;   // ceil(2^32 / TX): t / TX = (t tx_recip) >> 32 exactly for t, TX < 2^16
     unsigned long long* stats;   // diagnostics [8], see hr_scene_stats
@@ -840,7 +841,15 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
                 if (kImage) {
     #pragma unroll
                     for (int c = 0; c < 4; ++c)
-                        if (has_tile && y < P.H && x0 + c < P.W) {
+                        if (P.tiled) {
+                            float* o = img + 3 * ((size_t)(t * kG + gl) * 4 + c);
+                            const bool in = y < P.H && x0 + c < P.W;
+                            if (has_tile) {
+                                o[0] = in ? sh[c] * P.alb0 : 0.0f;
+                                o[1] = in ? sh[c] * P.alb1 : 0.0f;
+                                o[2] = in ? sh[c] * P.alb2 : 0.0f;
+                            }
+                        } else if (has_tile && y < P.H && x0 + c < P.W) {
                             const size_t q = (size_t)y * P.W + x0 + c;
                             if (ids) {
                                 ids[q] = bs[c] != INT_MAX ? __float_as_int(rec[bs[c]].shade) : -1;
@@ -941,6 +950,7 @@ __global__ void normals_kernel(const float* verts, const int32_t* tris, int nt, 
     tnrm[3 * t + 2] = (float)(n2 * inv);
 }
 
+// per tile the sum of its target's squares, rows first (target in tile order)
 __global__ void tile_t2_kernel(const float* target, int W, int H, int TX, int TH, int T, float* out) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= T) return;
@@ -950,7 +960,7 @@ __global__ void tile_t2_kernel(const float* target, int W, int H, int TX, int TH
         for (int xx = 0; xx < kTW; ++xx) {
             const int x = tx * kTW + xx, y = ty * TH + yy;
             if (x >= W || y >= H) continue;
-            const size_t p = (size_t)y * W + x;
+            const size_t p = ((size_t)t * 2 * TH + 2 * yy + (xx >> 2)) * 4 + (xx & 3);
             for (int c = 0; c < 3; ++c) s += target[3 * p + c] * target[3 * p + c];
         }
     out[t] = s;
@@ -961,6 +971,8 @@ __global__ void tile_t2_kernel(const float* target, int W, int H, int TX, int TH
 // tile's fixed work is a third of a 512x512 render's.  Together with the LOP3 above,
 // before -> after per estimate: 256x256, 4,096 renders 844 -> 793 us; 400x400, 512
 // renders 259 -> 220 us; 512x512, 256 renders 215 -> 189 us; 128x128 no change.
+// (A target rendered from parameters is written in this order by the raster; this
+// kernel lays out a caller's image.)
 // Lane l of a tile (row l / 2, columns 4 (l % 2) to
 // 4 (l % 2) + 3) has its 12 values together, 0 outside the image
 __global__ void target_tiles_kernel(const float* target, int W, int H, int TX, int TH, int n, float* out) {
@@ -986,6 +998,7 @@ RvArgs make_args(const DevScene& sc, bool compact = false, bool redo = false) {
     a.bytes = (int)sc.rv_smem;
     a.vreg = sc.rv_vreg;
     a.slots = sc.rv_cslots;
+    a.tiled = 0;
     a.redo = redo ? 1 : 0;
     a.stats = sc.rv_stats;
     return a;
@@ -1097,11 +1110,11 @@ void revolve_prepare(DevScene& sc, int max_smem, cudaStream_t s) {
     }
 }
 
-void revolve_tile_t2(DevScene& sc, cudaStream_t s) {
+void revolve_tables(DevScene& sc, const float* image, cudaStream_t s) {
     const int TX = (sc.W + kTW - 1) / kTW, TY = (sc.H + sc.rv_th - 1) / sc.rv_th;
     const int n = TX * TY * kTW * sc.rv_th;
-    target_tiles_kernel<<<(n + 255) / 256, 256, 0, s>>>(sc.target, sc.W, sc.H, TX, sc.rv_th, n, sc.rv_target);
-    tile_t2_kernel<<<(TX * TY + 127) / 128, 128, 0, s>>>(sc.target, sc.W, sc.H, TX, sc.rv_th, TX * TY, sc.tile_t2);
+    if (image) target_tiles_kernel<<<(n + 255) / 256, 256, 0, s>>>(image, sc.W, sc.H, TX, sc.rv_th, n, sc.rv_target);
+    tile_t2_kernel<<<(TX * TY + 127) / 128, 128, 0, s>>>(sc.rv_target, sc.W, sc.H, TX, sc.rv_th, TX * TY, sc.tile_t2);
 }
 
 int revolve_tiles(const DevScene& sc) {
@@ -1129,6 +1142,15 @@ void launch_revolve_loss(const DevScene& sc, const RenderBatch& b, cudaStream_t 
     auto kernel = sc.rv_th == 4 ? revolve_kernel<4, false, false> : revolve_kernel<8, false, false>;
     if (compact) kernel<<<grid, kThreads, sc.rv_smem, s>>>(a, b, nullptr, nullptr, nullptr);
     else launch_after(kernel, dim3(grid), dim3(kThreads), sc.rv_smem, s, a, b, nullptr, nullptr, nullptr);
+}
+
+// the target at params, in tile order
+void launch_revolve_target(const DevScene& sc, const float* params, cudaStream_t s) {
+    RenderBatch b{};
+    RvArgs a = make_args(sc);
+    a.tiled = 1;
+    auto kernel = sc.rv_th == 4 ? revolve_kernel<4, true, false> : revolve_kernel<8, true, false>;
+    kernel<<<1, kThreads, sc.rv_smem, s>>>(a, b, params, sc.rv_target, nullptr);
 }
 
 // one image at params: colours into img [H][W][3], or, with ids non-null,
