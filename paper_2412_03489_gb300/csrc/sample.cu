@@ -92,9 +92,11 @@ __device__ __forceinline__ void hessian_weights(const float* s_t, const double* 
         if (rem == 0) continue;
         const int j = i + rem;
         for (int r = r0; r < rows; r += rstep) {
-            const float2 c = s_c[r];   // is4 / S in two floats, 0 without a mixture density
+            // is4 / S in two floats (0 too where it underflows: wide bandwidths), 1/S, 0 without a mixture density
+            const float2 c = s_c[r];
+            const double iS = s_iS[r];
             wm[(size_t)r * E + e] =
-                c.x != 0.0f ? off_diagonal_weight(s_t[r * n + i], s_t[r * n + j], c.x, c.y, is4, s_iS[r]) : 0.0f;
+                iS != 0.0 ? off_diagonal_weight(s_t[r * n + i], s_t[r * n + j], c.x, c.y, is4, iS) : 0.0f;
         }
     }
     for (int x = threadIdx.x; x < rows * n; x += blockDim.x) {

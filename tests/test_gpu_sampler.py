@@ -117,3 +117,17 @@ def test_many_draws_equal_the_oracles(quantity, strategy):
     ref = O.estimate(O.FunctionRenderer(lambda P: np.zeros(len(P)), 2), quantity, sc["theta_query"], sc["sigma"], 8192,
                      strategy, 3, 4, sub=5)
     assert np.array_equal(d["tau"], ref.tau)
+
+
+@pytest.mark.parametrize("n", [2, 16, 33])
+@pytest.mark.parametrize("sigma", [1e-15, 1e-6, 1e9, 2e11, 3e11, 1e12, 1e18])
+def test_weights_at_extreme_bandwidths(n, sigma):
+    """Aggregate Hessian weights are of the order of 1 / sigma^2, a normal float here, although
+    sigma^-4 is not one for the larger bandwidths (or for the smallest)."""
+    sc = dict(scene(n), sigma=sigma)
+    M = 2 * 21
+    _, d, _ = run(sc, "hessian", "aggregate", M)
+    ref = O.estimate(O.FunctionRenderer(lambda P: np.zeros(len(P)), n), "hessian", sc["theta_query"], sigma, M,
+                     "aggregate", 3, 4, sub=5)
+    assert np.array_equal(d["tau"], ref.tau)
+    assert np.allclose(d["w"], ref.w.astype(np.float32), rtol=2e-7, atol=2e-7 * np.abs(ref.w).max())
