@@ -601,8 +601,8 @@ hr_status hr_profile_last(hr_scene scene, float* ms3);
 /* ---------------------------------------------------------------------------
  * Autotuning of launch shapes.  Each scene kind has render+loss launch-shape
  * variants (path tracer, where one CTA renders one perturbation: resident
- * CTAs per SM, i.e. register caps, by the launch's size, 3 or 2; disc and
- * squares: 8 / 4 / 16 warps per CTA, one warp per
+ * CTAs per SM, i.e. register caps, 2 to 4 by the launch's size, 2 to 3 or 2;
+ * disc and squares: 8 / 4 / 16 warps per CTA, one warp per
  * perturbation; mesh and 2D triangles: one shape) and the sampler runs with
  * 16, 32, 64 or 128 threads per block (16 spreads small requests over more
  * SMs; with 64 or 128, a block takes its aggregate Hessian pairs diagonal-lobe
@@ -613,7 +613,9 @@ hr_status hr_profile_last(hr_scene scene, float* ms3);
  * max(n_probe, 8 x the SM count) perturbations at h_theta [n] (v = ones,
  * sigma 0.05; median of 3 after a warm-up; the floor keeps the GPU full so
  * that occupancy shows), keeps the fastest for the scene and, if info is not NULL,
- * reports the choice and the timings (ms).  hr_set_tuning sets a choice
+ * reports the choice and the timings (ms).  Where such a path-traced estimate
+ * renders pairs of perturbations per CTA, which has one shape, the render variant
+ * stays 0 and one timing stands for all.  hr_set_tuning sets a choice
  * directly (HR_ERR_INVALID_ARG when out of range).  Scenes start at variant 0
  * and 32 sampler threads.
  * ------------------------------------------------------------------------- */

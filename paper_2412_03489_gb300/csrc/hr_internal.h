@@ -240,6 +240,18 @@ struct DevScene {
 
 // launch-shape variants of a scene kind's render+loss kernel (1 = none)
 int render_variant_count(int kind);
+// do M perturbations of one estimate take a kernel that has these variants?
+bool ptbox_variants_apply(const DevScene& sc, int M);
+
+// Resident CTAs per SM of the path tracer's kernel with one render per CTA: as many
+// as the launch has, 2 to 4 (fewer leave each its registers; 24x24, M = 64: 31 us with
+// 2, 35 with 3, 38 with 4; M = 1,024: 101 with 3, 89 with 4).  Variants 1 and 2 cap it
+// at 3 and 2: tuned on a launch that fills the GPU, they hold for such launches
+// only, and smaller ones keep their shape.
+inline int ptbox_resident(int variant, int M, int sms) {
+    const int by_size = M <= 2 * sms ? 2 : M <= 3 * sms ? 3 : 4, cap = 4 - variant;
+    return by_size < cap ? by_size : cap;
+}
 
 // shared-memory layout and tile height of one mesh render on a device with
 // max_smem bytes of opt-in shared memory per block (sets rv_smem, rv_vreg,

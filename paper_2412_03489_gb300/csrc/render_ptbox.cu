@@ -1125,12 +1125,7 @@ void launch_loss(const DevScene& sc, const RenderBatch& b, cudaStream_t s) {
         launch_pairs(a, b, p, s);
         return;
     }
-    // variant 0: as many resident CTAs per SM as the launch has, 2 to 4 (fewer
-    // leave each its registers; 24x24, M = 64: 31 us with 2, 35 with 3, 38 with 4;
-    // M = 1,024: 101 with 3, 89 with 4)
-    const int shape = sc.render_variant == 1 ? 3 : sc.render_variant == 2 ? 2
-                      : b.M <= 2 * num_sms() ? 2 : b.M <= 3 * num_sms() ? 3 : 4;
-    switch (shape) {
+    switch (ptbox_resident(sc.render_variant, b.M, num_sms())) {
         case 2: ptbox_kernel<false, 2, kCanon><<<b.M, kThreads, 0, s>>>(a, b, nullptr, 0, 0, 0, 0, 0, 0, nullptr); break;
         case 3: ptbox_kernel<false, 3, kCanon><<<b.M, kThreads, 0, s>>>(a, b, nullptr, 0, 0, 0, 0, 0, 0, nullptr); break;
         default: ptbox_kernel<false, 4, kCanon><<<b.M, kThreads, 0, s>>>(a, b, nullptr, 0, 0, 0, 0, 0, 0, nullptr); break;
@@ -1141,12 +1136,18 @@ void launch_loss(const DevScene& sc, const RenderBatch& b, cudaStream_t s) {
 
 // Launch-shape variants (autotuner) of the kernel of one render per CTA: the same
 // 256-thread layout and arithmetic, different register caps through the minimum
-// number of resident CTAs per SM (by the launch's size, 3, 2), so the choice
-// never changes a result.  Scenes with the procedural box's quad layout use the
-// compile-time-axis intersection, and the pair kernel where it is faster.
+// number of resident CTAs per SM (ptbox_resident: by the launch's size, that up to 3,
+// up to 2), so the choice never changes a result.  Scenes with the procedural box's
+// quad layout use the compile-time-axis intersection, and the pair kernel, which has
+// one shape, where it is faster.
 void launch_ptbox_loss(const DevScene& sc, const RenderBatch& b, cudaStream_t s) {
     if (canonical_axes(sc)) launch_loss<true>(sc, b, s);
     else launch_loss<false>(sc, b, s);
+}
+
+bool ptbox_variants_apply(const DevScene& sc, int M) {
+    if (sc.count_work && sc.pt_stats) return false;
+    return !canonical_axes(sc) || (M & 1) || pair_shape(sc.W * sc.H, M / 2, num_sms()).parts == 0;
 }
 
 cudaError_t ptbox_prepare() {

@@ -15,7 +15,7 @@ namespace hr {
 
 int render_variant_count(int kind) {
     switch (kind) {
-        case HR_SCENE_PTBOX: return 3;     // one render per CTA: resident CTAs per SM by the launch, 3, 2 (register caps 64 to 128)
+        case HR_SCENE_PTBOX: return 3;     // one render per CTA: resident CTAs per SM by the launch, at most 3, at most 2
         case HR_SCENE_DISC2D: return 3;    // 8 / 4 / 16 warps per CTA, one warp per perturbation
         case HR_SCENE_BOXES2D: return 3;
         default: return 1;                 // mesh and 2D triangles: one CTA shape
@@ -93,8 +93,16 @@ hr_status hr_autotune(hr_scene s, const double* h_theta, int32_t n_probe, hr_tun
     rep.n_render_variants = nv;
     rep.n_sample_variants = 4;
     hr_status st = HR_OK;
+    // A path-traced probe may take the kernel of pairs, which has no variants: all
+    // three are then one launch, timed once, and the choice stays at variant 0
+    // (picked by noise, it would pin the other kernel's launches of this scene).
+    const bool choice = s->sc.kind != HR_SCENE_PTBOX || ptbox_variants_apply(s->sc, probe_m);
     int best_v = 0;
     for (int k = 0; k < nv && st == HR_OK; ++k) {
+        if (k > 0 && !choice) {
+            rep.render_ms[k] = rep.render_ms[0];
+            continue;
+        }
         s->sc.render_variant = k;
         st = probe(s, h_theta, v.data(), o, 1, 3, &rep.render_ms[k]);
         if (st == HR_OK && rep.render_ms[k] < rep.render_ms[best_v]) best_v = k;

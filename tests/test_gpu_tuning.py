@@ -59,3 +59,16 @@ def test_out_of_range_settings_are_rejected():
     with pytest.raises(hr.HRError, match="status -1"):
         hr.hr_autotune(S.handle, sc["theta_query"], 3)
     S.close()
+
+
+@pytest.mark.parametrize("width,height", [(32, 32), (48, 48), (64, 64)])
+def test_no_choice_among_equal_launches(width, height):
+    """From 1,024 pixels a probe of the path tracer takes the kernel of pairs whatever the
+    variant: the tuner keeps variant 0 and reports one timing (three medians of
+    separately timed launches do not agree to the bit)."""
+    sc = wl.ptbox_scene(width=width, height=height, spp=1, target_spp=1)
+    S = hr.Scene(sc)
+    info = hr.hr_autotune(S.handle, sc["theta_query"], 2048)
+    assert info.render_variant == 0 and info.n_render_variants == 3
+    assert info.render_ms[0] > 0 and len(set(info.render_ms[:3])) == 1
+    S.close()
