@@ -27,6 +27,31 @@ __global__ void __launch_bounds__(32 * kW) disc_loss_kernel(RenderBatch b, int W
     if (lane == 0) *pt.loss = loss;
 }
 
+// The same losses against a target that is not binary, for larger images: every
+// pixel is visited, so the centres are read from shared memory, and the next
+// kernel may start only when this one's work begins (let start at once, the next
+// call's renders are placed while these run, unevenly over the SMs: 1,024 renders of
+// 333x250 in 152 us instead of 93).  Aggregate Hessians in us, from the table in
+// global memory and so: 333x250, 64 renders 179, 90; 1,024 204, 93; 16,384
+// 1,173, 984; 512x512, 1,024 renders 355, 205.
+template <int kW>
+__global__ void __launch_bounds__(32 * kW) disc_grey_kernel(RenderBatch b, int W, int H, float radius,
+                                                            const float* __restrict__ target) {
+    __shared__ float s_px[HR_MAX_IMAGE_SIDE], s_py[HR_MAX_IMAGE_SIDE];
+    centre_tables(s_px, s_py, W, H);
+    __syncthreads();
+    wait_for_previous();
+    let_next_start();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int m = blockIdx.x * kW + warp;
+    if (m >= b.M) return;
+    const Pert pt = resolve(b, m);
+    const float cx = __fadd_rn(pt.theta[0], pt.tau[0]);
+    const float cy = __fadd_rn(pt.theta[1], pt.tau[1]);
+    const float loss = disc_loss_warp(target, DiscBits{}, W, H, radius, s_px, s_py, cx, cy, lane);
+    if (lane == 0) *pt.loss = loss;
+}
+
 // Bit-packed target rows (bit x % 32 of word x / 32 of row y: pixel (x, y) is
 // 1), found[0] raised by any pixel other than 0 or 1, found[1] counting the ones.
 __global__ void disc_bits_kernel(const float* __restrict__ target, int W, int H, int words, uint32_t* bits,
@@ -127,12 +152,24 @@ void launch_boxes_image(const DevScene& sc, const float* params, float* img, cud
     boxes_image_kernel<<<(npx + 255) / 256, 256, 0, s>>>(params, sc.n / 2, sc.W, sc.H, sc.radius, img);
 }
 
+template <int kW>
+void launch_disc_as(const DevScene& sc, const RenderBatch& b, cudaStream_t s) {
+    const dim3 grid((b.M + kW - 1) / kW), block(32 * kW);
+    // up to 64x64 filling the shared tables takes what reading them saves (64x64, 64 / 1,024 /
+    // 16,384 renders: 12.0 / 12.9 / 32.7 us from the table, 12.9 / 13.5 / 33.8 so; 80x80: 21.8 / 25.0 /
+    // 102.6, 13.8 / 14.4 / 91.2)
+    if (!sc.tbinary && sc.W * sc.H > 4096)
+        launch_after(disc_grey_kernel<kW>, grid, block, 0, s, b, sc.W, sc.H, sc.radius, sc.target);
+    else
+        launch_after(disc_loss_kernel<kW>, grid, block, 0, s, b, sc.W, sc.H, sc.radius, sc.target, sc.centres,
+                     DiscBits{sc.tbinary ? sc.tbits : nullptr, sc.tpre, sc.tones});
+}
+
 void launch_disc_loss(const DevScene& sc, const RenderBatch& b, cudaStream_t s) {
-    const DiscBits tb{sc.tbinary ? sc.tbits : nullptr, sc.tpre, sc.tones};
     switch (sc.render_variant) {
-        case 1: launch_after(disc_loss_kernel<4>, dim3((b.M + 3) / 4), dim3(128), 0, s, b, sc.W, sc.H, sc.radius, sc.target, sc.centres, tb); break;
-        case 2: launch_after(disc_loss_kernel<16>, dim3((b.M + 15) / 16), dim3(512), 0, s, b, sc.W, sc.H, sc.radius, sc.target, sc.centres, tb); break;
-        default: launch_after(disc_loss_kernel<8>, dim3((b.M + 7) / 8), dim3(256), 0, s, b, sc.W, sc.H, sc.radius, sc.target, sc.centres, tb); break;
+        case 1: launch_disc_as<4>(sc, b, s); break;
+        case 2: launch_disc_as<16>(sc, b, s); break;
+        default: launch_disc_as<8>(sc, b, s); break;
     }
 }
 
