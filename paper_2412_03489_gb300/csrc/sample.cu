@@ -466,9 +466,11 @@ void launch_sample(const SampleArgs& a, int n_groups, int max_P, cudaStream_t s)
     const size_t per_pair = 2 * (size_t)a.n * (sizeof(double) + sizeof(float));
     int np = legs / 2;
     while (np > 1 && np * per_pair > 40 * 1024) np /= 2;
-    // launches bound by the FP64 rate: enough pairs that the Gaussian units fill
-    // their warps (one dim in two of 16 pairs leaves half a warp idle)
-    if (np == 16 && (a.n & 3) == 2 && (int64_t)n_groups * max_P >= 32 * 8 * num_sms() && 32 * per_pair <= 40 * 1024)
+    // launches bound by the FP64 rate: enough pairs that the Gaussian units, a lane
+    // per two dims of a pair, fill their warps (16 pairs of an odd number of such
+    // lanes leave half a warp idle).  131,072 renders, 16 and 32 pairs, us per estimate:
+    // plain gradient of 1 dim 76.8, 71.7, aggregate of 9 dims 260, 244, of 13 324, 306.
+    if (np == 16 && (((a.n + 1) / 2) & 1) && (int64_t)n_groups * max_P >= 32 * 8 * num_sms() && 32 * per_pair <= 40 * 1024)
         np = 32;
     // many dims: spread few pairs over the SMs
     while (np > 2 && a.n >= 16 && (int64_t)n_groups * ((max_P + np - 1) / np) < num_sms()) np /= 2;

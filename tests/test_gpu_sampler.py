@@ -3,6 +3,7 @@ launches change: dims per warp, ragged last blocks, many weights per row, rows
 per chunk."""
 import numpy as np
 import pytest
+import torch
 
 import oracle as O
 from paper_2412_03489_gb300 import build as hb
@@ -131,3 +132,19 @@ def test_weights_at_extreme_bandwidths(n, sigma):
                      "aggregate", 3, 4, sub=5)
     assert np.array_equal(d["tau"], ref.tau)
     assert np.allclose(d["w"], ref.w.astype(np.float32), rtol=2e-7, atol=2e-7 * np.abs(ref.w).max())
+
+
+@pytest.mark.parametrize("n", [1, 2, 4, 5, 6, 13, 33])
+def test_large_launches_equal_the_other_shapes(n):
+    """Launches large enough that a block takes 32 pairs (an odd number of dim pairs), with a
+    ragged last block: the bits of the shapes with 8 and 64 pairs a block."""
+    sc = scene(n)
+    s, M = hr.Scene(sc), 2 * (256 * torch.cuda.get_device_properties(0).multi_processor_count + 37)
+    v = np.random.default_rng(7).normal(size=n)
+    outs = {}
+    for legs in (32, 16, 128):
+        hr.hr_set_tuning(s.handle, 0, legs)
+        outs[legs] = [s.estimate(q, sc["theta_query"], sc["sigma"], M, st, 3, 4, v=v if q == hr.HR_HVP else None)
+                      for q in (hr.HR_GRAD, hr.HR_HVP) for st in (hr.HR_AGGREGATE, hr.HR_PLAIN)]
+    s.close()
+    assert all(np.array_equal(a, b) for legs in (16, 128) for a, b in zip(outs[32], outs[legs]))
