@@ -92,11 +92,9 @@ __device__ __forceinline__ void hessian_weights(const float* s_t, const double* 
         if (rem == 0) continue;
         const int j = i + rem;
         for (int r = r0; r < rows; r += rstep) {
-            // is4 / S in two floats (0 too where it underflows: wide bandwidths), 1/S, 0 without a mixture density
-            const float2 c = s_c[r];
-            const double iS = s_iS[r];
+            const float2 c = s_c[r];   // is4 / S in two floats, 0 without a mixture density
             wm[(size_t)r * E + e] =
-                iS != 0.0 ? off_diagonal_weight(s_t[r * n + i], s_t[r * n + j], c.x, c.y, is4, iS) : 0.0f;
+                c.x != 0.0f ? off_diagonal_weight(s_t[r * n + i], s_t[r * n + j], c.x, c.y, is4, s_iS[r]) : 0.0f;
         }
     }
     for (int x = threadIdx.x; x < rows * n; x += blockDim.x) {
@@ -265,7 +263,10 @@ __global__ void __launch_bounds__(kSampleThreads) sample_kernel(SampleArgs a, Lo
         s_iS[r] = iS;
         s_tv[r] = tv;
         const double c = L.is4 * iS;
-        s_c[r] = make_float2((float)c, (float)(c - (double)(float)c));
+        const float ch = (float)c;
+        // (0 says that there is no density: a product that leaves FP32 becomes the smallest
+        // number instead, with which the weights take their FP64 form)
+        s_c[r] = make_float2(ch != 0.0f || iS == 0.0 ? ch : 0x1p-149f, (float)(c - (double)ch));
     }
     if (!a.w || G.quantity == 3) return;
     __syncthreads();
