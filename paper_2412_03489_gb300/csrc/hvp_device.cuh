@@ -30,7 +30,10 @@ __device__ __forceinline__ void hvp_product(HvpTile& S, const float* __restrict_
                                             const float* __restrict__ loss, int M, int n, const double* p, double is2,
                                             double is4, double* q, F beside) {
     const int ld = n | 1, tile = min(HvpTile::kRows, HvpTile::kDoubles / ld);
-    const uint32_t recip = (uint32_t)(((1u << 20) + (uint32_t)n - 1u) / (uint32_t)n);   // i / n for i < 2^15, n <= 64
+    // i / n = (i recip) >> 20 for the tile's i < rows n <= kDoubles: recip n - 2^20 < n <= 64, so the
+    // quotient is exact while i 63 < 2^20, and i recip <= rows (2^20 + n) stays within 32 bits
+    const uint32_t recip = (uint32_t)(((1u << 20) + (uint32_t)n - 1u) / (uint32_t)n);
+    static_assert(HvpTile::kDoubles * 63 < (1 << 20) && HvpTile::kRows < (1 << 11), "division by n");
     Kahan acc;
     if (threadIdx.x < n) S.p2[threadIdx.x] = p[threadIdx.x] * is2;
     for (int m0 = 0; m0 < M; m0 += tile) {
