@@ -609,9 +609,10 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
                 bool hit = true;
 #pragma unroll
                 for (int i = 0; i < 3; ++i) hit = hit && !(fmaf(A[i], A[i] > 0.0f ? fx1 : fx0, rt[i]) < neg[i]);
+                mask >>= 1;   // (in at the top, shifted down at the end: no shift by a variable)
                 if (hit) {
                     atomicAdd(cell, 1);
-                    mask |= (Mask)1 << bit;
+                    mask |= (Mask)1 << (8 * (int)sizeof(Mask) - 1);
                 }
                 left += (float)kTW;
                 ++cell;
@@ -622,6 +623,7 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
                     row_terms();
                 }
             }
+            mask >>= 8 * (int)sizeof(Mask) - rect;
             if constexpr (kCompact) tm16[k] = (uint16_t)mask;
             else tmask[k] = mask;
         }
@@ -642,6 +644,7 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
         // tiles are rastered together: every pixel's decisions are the same.
         const bool banded = !kCompact && total > cap;
         const int capb = banded ? cap - P.TY : cap;
+        const bool many_bands = banded && total > 4 * capb;
         int* rowtot = reinterpret_cast<int*>(ent) + capb;
         if (banded) {
             for (int r = warp; r < P.TY; r += kW) {
@@ -682,32 +685,51 @@ revolve_kernel(RvArgs P, RenderBatch b, const float* __restrict__ img_params, fl
                     const int nx = tx1 - tx0 + 1, rect = nx * (ty1 - ty0 + 1);
                     const int ya = max(ty0, r0), yb = min(ty1, r1 - 1);
                     if (ya > yb) continue;
-                    // columns of the first and rows outside the box in the last tiles, as bits
+                    // columns and rows outside the box in the first and last tiles, as bits (row bits
+                    // >= kTH are never tested)
                     const uint32_t out_l = ~(0xFFu << (xlo & 7)) & 0xFFu, out_r = (0xFEu << (xhi & 7)) & 0xFFu;
+                    const uint32_t out_t = (~(0xFFu << (ylo - ty0 * kTH)) & 0xFFu) << 8;
+                    const uint32_t out_b = ((0xFEu << (yhi - ty1 * kTH)) & 0xFFu) << 8;
                     auto put = [&](int ty, int tx) {
                         const uint32_t cols = (tx == tx0 ? out_l : 0u) | (tx == tx1 ? out_r : 0u);
-                        const uint32_t rows = span_bits(ylo - ty * kTH, yhi - ty * kTH);   // bits >= kTH are never tested
-                        ent[atomicAdd(&tcnt[ty * P.TX + tx], 1)] = ((uint32_t)k << 16) | ((~rows & 0xFFu) << 8) | cols;
+                        const uint32_t rows = (ty == ty0 ? out_t : 0u) | (ty == ty1 ? out_b : 0u);
+                        ent[atomicAdd(&tcnt[ty * P.TX + tx], 1)] = ((uint32_t)k << 16) | rows | cols;
                     };
                     if (rect > (kCompact ? 16 : 64)) {
                         for (int ty = ya; ty <= yb; ++ty)
                             for (int tx = tx0; tx <= tx1; ++tx) put(ty, tx);
                         continue;
                     }
+                    // Where a band holds few of a rectangle's rows, its tiles in turn: neighbouring
+                    // survivors then write neighbouring tiles together (fewer conflicts, here and on
+                    // the records in the raster).  14 stacked sheets of 8x8 quads at 512x512, eleven
+                    // bands, 1,024 renders: 8.92 ms, by set bits 9.20; 8 sheets at 256x256, two
+                    // bands: 1.35, 1.32; at 128x128, one band: 0.607, 0.590.
+                    if (!kCompact && many_bands) {
+                        unsigned long long mask = tmask[k] >> ((ya - ty0) * nx);
+                        int ty = ya, tx = tx0;
+                        for (int q = (yb + 1 - ya) * nx; q > 0; --q, mask >>= 1) {
+                            if (mask & 1ull) put(ty, tx);
+                            if (++tx > tx1) { tx = tx0; ++ty; }
+                        }
+                        continue;
+                    }
                     // the mask's set bits, lowest first; row of bit b: b / nx (exact for b, nx <= 64)
                     const uint32_t recip = (65536u + (uint32_t)nx - 1u) / (uint32_t)nx;
-                    if constexpr (kCompact) {
-                        for (uint32_t mask = tm16[k]; mask; mask &= mask - 1u) {
-                            const uint32_t bit = (uint32_t)__ffs((int)mask) - 1u, row = (bit * recip) >> 16;
+                    auto put_bits = [&](uint32_t mask, uint32_t from) {
+                        for (; mask; mask &= mask - 1u) {
+                            const uint32_t bit = (uint32_t)__ffs((int)mask) + from, row = (bit * recip) >> 16;
                             put(ty0 + (int)row, tx0 + (int)(bit - row * (uint32_t)nx));
                         }
+                    };
+                    if constexpr (kCompact) {
+                        put_bits(tm16[k], ~0u);
                     } else {
-                        unsigned long long mask = tmask[k];
-                        for (; mask; mask &= mask - 1ull) {
-                            const uint32_t bit = (uint32_t)__ffsll((long long)mask) - 1u, row = (bit * recip) >> 16;
-                            const int ty = ty0 + (int)row;
-                            if (ty >= ya && ty <= yb) put(ty, tx0 + (int)(bit - row * (uint32_t)nx));
-                        }
+                        // only the bits of the band's rows, 0 <= first < end <= 64
+                        const int first = (ya - ty0) * nx, end = (yb + 1 - ty0) * nx;
+                        const unsigned long long mask = tmask[k] & (~0ull << first) & (~0ull >> (64 - end));
+                        put_bits((uint32_t)mask, ~0u);
+                        put_bits((uint32_t)(mask >> 32), 31u);
                     }
                 }
             }

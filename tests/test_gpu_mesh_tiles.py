@@ -44,3 +44,17 @@ def test_a_smaller_scene_made_later_leaves_a_larger_one_its_launches():
     for S in scenes + [late]:
         S.close()
     assert all(np.array_equal(a, b) for a, b in zip(after, before))
+
+
+@pytest.mark.parametrize("layers,grid,size", [(8, 8, 128), (8, 8, 256), (14, 8, 256), (8, 8, 512), (14, 8, 512), (12, 4, 300)])
+def test_stacked_sheets(layers, grid, size):
+    """Every triangle faces the camera and every tile is many layers deep: bins filled at
+    once, in a few bands of tile rows and in many, loss by loss (tolerance as above)."""
+    sc = wl.revolve_scene(width=size, height=size)
+    sc["vertices"], sc["triangles"] = wl.sheets_mesh(layers, grid)
+    S, r = hr.Scene(sc), O.RevolveRenderer(sc)
+    th = np.asarray(sc["theta_query"], np.float64)
+    _, d = S.estimate(hr.HR_HESSIAN, th, 0.1, 4, hr.HR_AGGREGATE, 3, 4, debug=True)
+    S.close()
+    want = np.array([r.loss(th.astype(np.float32) + t, None) for t in d["tau"]])
+    np.testing.assert_allclose(d["losses"], want, rtol=2e-5)
