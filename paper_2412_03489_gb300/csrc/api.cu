@@ -110,11 +110,14 @@ using namespace hr;
 
 namespace {
 
+// A scene's copies go on its own stream, whose kernels read them: cudaMemcpy from
+// pageable memory may return before the data has arrived, and a non-blocking stream
+// does not wait for it.
 template <class T>
-cudaError_t upload(T** dst, const T* src, size_t count) {
+cudaError_t upload(T** dst, const T* src, size_t count, cudaStream_t s) {
     cudaError_t e = cudaMalloc((void**)dst, sizeof(T) * (count ? count : 1));
     if (e != cudaSuccess) return e;
-    if (count) e = cudaMemcpy(*dst, src, sizeof(T) * count, cudaMemcpyHostToDevice);
+    if (count) e = cudaMemcpyAsync(*dst, src, sizeof(T) * count, cudaMemcpyHostToDevice, s);
     return e;
 }
 
@@ -466,8 +469,8 @@ hr_status hr_create_scene(const hr_scene_desc* d, hr_scene* out) {
                 return fail(HR_ERR_UNSUPPORTED, "mesh of %d triangles at %dx%d does not fit in %d B of shared memory",
                             sc.nt, sc.W, sc.H, maxsm);
             }
-            if ((e = upload(&sc.verts, d->vertices, 3 * (size_t)sc.nv)) != cudaSuccess) return bail(e, "vertices");
-            if ((e = upload(&sc.tris, d->triangles, 3 * (size_t)sc.nt)) != cudaSuccess) return bail(e, "triangles");
+            if ((e = upload(&sc.verts, d->vertices, 3 * (size_t)sc.nv, s->stream)) != cudaSuccess) return bail(e, "vertices");
+            if ((e = upload(&sc.tris, d->triangles, 3 * (size_t)sc.nt, s->stream)) != cudaSuccess) return bail(e, "triangles");
             // one allocation: target in tile order | counters | sums by tile | normals
             const size_t tiles = revolve_tiles(sc), n_target = 3 * 8 * (size_t)sc.rv_th * tiles;
             const size_t n_stats = 8 * sizeof(unsigned long long) / sizeof(float);
@@ -483,8 +486,8 @@ hr_status hr_create_scene(const hr_scene_desc* d, hr_scene* out) {
         }
         case HR_SCENE_TRIS2D:
             sc.n_tris = d->n_tris;
-            if ((e = upload(&sc.raw, d->raw_params, 9 * (size_t)sc.n_tris)) != cudaSuccess) return bail(e, "raw");
-            if ((e = upload(&sc.pidx, d->param_index, (size_t)sc.n)) != cudaSuccess) return bail(e, "param_index");
+            if ((e = upload(&sc.raw, d->raw_params, 9 * (size_t)sc.n_tris, s->stream)) != cudaSuccess) return bail(e, "raw");
+            if ((e = upload(&sc.pidx, d->param_index, (size_t)sc.n, s->stream)) != cudaSuccess) return bail(e, "param_index");
             break;
         case HR_SCENE_PTBOX:
             for (int q = 0; q < 12; ++q) {
@@ -501,11 +504,11 @@ hr_status hr_create_scene(const hr_scene_desc* d, hr_scene* out) {
             for (int c = 0; c < 3; ++c) sc.emission[c] = d->emission[c];
             sc.spp = d->spp; sc.target_spp = d->target_spp; sc.depth = d->depth; sc.scene_seed = d->seed;
             if ((e = cudaMalloc(&sc.pt_stats, 4 * sizeof(unsigned long long))) != cudaSuccess) return bail(e, "stats");
-            if ((e = cudaMemset(sc.pt_stats, 0, 4 * sizeof(unsigned long long))) != cudaSuccess) return bail(e, "stats");
+            if ((e = cudaMemsetAsync(sc.pt_stats, 0, 4 * sizeof(unsigned long long), s->stream)) != cudaSuccess) return bail(e, "stats");
             break;
         case HR_SCENE_QUADRATIC:
-            if ((e = upload(&sc.qA, d->quad_A, (size_t)sc.n * sc.n)) != cudaSuccess) return bail(e, "A");
-            if ((e = upload(&sc.qb, d->quad_b, (size_t)sc.n)) != cudaSuccess) return bail(e, "b");
+            if ((e = upload(&sc.qA, d->quad_A, (size_t)sc.n * sc.n, s->stream)) != cudaSuccess) return bail(e, "A");
+            if ((e = upload(&sc.qb, d->quad_b, (size_t)sc.n, s->stream)) != cudaSuccess) return bail(e, "b");
             break;
         case HR_SCENE_NEGGAUSS:
             sc.gauss_sigma = d->gauss_sigma;
@@ -513,22 +516,23 @@ hr_status hr_create_scene(const hr_scene_desc* d, hr_scene* out) {
     }
     if (analytic) {
         // no target: the loss is f itself
-        if ((e = cudaMemset(sc.target, 0, sizeof(float) * npx)) != cudaSuccess) return bail(e, "target");
+        if ((e = cudaMemsetAsync(sc.target, 0, sizeof(float) * npx, s->stream)) != cudaSuccess) return bail(e, "target");
     } else if (d->target_image && mesh) {
         float* image = nullptr;
-        if ((e = upload(&image, d->target_image, npx)) != cudaSuccess) return bail(e, "target upload");
+        if ((e = upload(&image, d->target_image, npx, s->stream)) != cudaSuccess) return bail(e, "target upload");
         revolve_tables(sc, image, s->stream);
         e = cudaStreamSynchronize(s->stream);
         cudaFree(image);
         if (e != cudaSuccess) return bail(e, "target tiles");
     } else if (d->target_image) {
-        if ((e = cudaMemcpy(sc.target, d->target_image, sizeof(float) * npx, cudaMemcpyHostToDevice)) != cudaSuccess)
+        if ((e = cudaMemcpyAsync(sc.target, d->target_image, sizeof(float) * npx, cudaMemcpyHostToDevice, s->stream)) !=
+            cudaSuccess)
             return bail(e, "target upload");
     } else {
         std::vector<float> p32(sc.n);
         for (int i = 0; i < sc.n; ++i) p32[i] = (float)d->theta_target[i];
         float* dp = nullptr;
-        if ((e = upload(&dp, p32.data(), (size_t)sc.n)) != cudaSuccess) return bail(e, "target params");
+        if ((e = upload(&dp, p32.data(), (size_t)sc.n, s->stream)) != cudaSuccess) return bail(e, "target params");
         if (mesh) {
             launch_revolve_target(sc, dp, s->stream);
             revolve_tables(sc, nullptr, s->stream);
@@ -694,7 +698,7 @@ hr_status hr_render_ids(hr_scene s, const double* h_params, int32_t* h_ids) {
     if (s->ws.render_img.reserve(sizeof(int32_t) * npx) != cudaSuccess ||
         s->ws.render_params.reserve(sizeof(p32)) != cudaSuccess)
         return fail(HR_ERR_OOM, "render buffers");
-    cudaError_t e = cudaMemcpy(s->ws.render_params.ptr, p32, sizeof(p32), cudaMemcpyHostToDevice);
+    cudaError_t e = cudaMemcpyAsync(s->ws.render_params.ptr, p32, sizeof(p32), cudaMemcpyHostToDevice, s->stream);
     if (e != cudaSuccess) return fail(HR_ERR_CUDA, "params: %s", cudaGetErrorString(e));
     launch_revolve_image(sc, (const float*)s->ws.render_params.ptr, nullptr, (int32_t*)s->ws.render_img.ptr, s->stream);
     if ((e = cudaGetLastError()) != cudaSuccess) return fail(HR_ERR_CUDA, "render: %s", cudaGetErrorString(e));
@@ -719,7 +723,8 @@ hr_status hr_render(hr_scene s, const double* h_params, uint64_t seed, uint32_t 
     if (s->ws.render_img.reserve(sizeof(float) * npx) != cudaSuccess ||
         s->ws.render_params.reserve(sizeof(float) * sc.n) != cudaSuccess)
         return fail(HR_ERR_OOM, "render buffers");
-    cudaError_t e = cudaMemcpy(s->ws.render_params.ptr, p32.data(), sizeof(float) * sc.n, cudaMemcpyHostToDevice);
+    cudaError_t e = cudaMemcpyAsync(s->ws.render_params.ptr, p32.data(), sizeof(float) * sc.n, cudaMemcpyHostToDevice,
+                                    s->stream);
     if (e != cudaSuccess) return fail(HR_ERR_CUDA, "params: %s", cudaGetErrorString(e));
     launch_render_image(sc, (const float*)s->ws.render_params.ptr, seed, request, sub, k, tag, spp,
                         (float*)s->ws.render_img.ptr, s->stream);

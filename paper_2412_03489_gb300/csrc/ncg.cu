@@ -330,7 +330,9 @@ hr_status hr_ncg_create(hr_scene scene, int32_t B, const double* theta0, const h
         (e = cudaMemset(st->rr.ptr, 0, sizeof(double) * B)) != cudaSuccess ||
         (e = cudaMemset(st->it.ptr, 0, sizeof(int32_t) * B)) != cudaSuccess ||
         (e = cudaMemset(st->ls.ptr, 0, sizeof(int32_t) * B)) != cudaSuccess ||
-        (e = cudaMemcpy(st->evc.ptr, &zero, sizeof(int32_t), cudaMemcpyHostToDevice)) != cudaSuccess) {
+        (e = cudaMemcpy(st->evc.ptr, &zero, sizeof(int32_t), cudaMemcpyHostToDevice)) != cudaSuccess ||
+        // (a copy or a fill may return before it has happened; the state's stream does not wait for this one)
+        (e = cudaStreamSynchronize(cudaStreamLegacy)) != cudaSuccess) {
         hr_ncg_destroy(st);
         return fail(HR_ERR_CUDA, "optimiser state upload: %s", cudaGetErrorString(e));
     }

@@ -270,7 +270,9 @@ hr_status hr_optstate_create(hr_scene scene, int32_t B, const double* theta0, co
     if ((e = cudaMemcpy(st->groups.ptr, groups.data(), sizeof(SampleGroup) * groups.size(), cudaMemcpyHostToDevice)) !=
             cudaSuccess ||
         (e = cudaMemcpy(st->theta.ptr, theta0, sizeof(double) * B * n, cudaMemcpyHostToDevice)) != cudaSuccess ||
-        (e = cudaMemcpy(st->step.ptr, &zero, sizeof(int32_t), cudaMemcpyHostToDevice)) != cudaSuccess) {
+        (e = cudaMemcpy(st->step.ptr, &zero, sizeof(int32_t), cudaMemcpyHostToDevice)) != cudaSuccess ||
+        // (a copy or a fill may return before it has happened; the state's stream does not wait for this one)
+        (e = cudaStreamSynchronize(cudaStreamLegacy)) != cudaSuccess) {
         hr_optstate_destroy(st);
         return fail(HR_ERR_CUDA, "optimizer state upload: %s", cudaGetErrorString(e));
     }
