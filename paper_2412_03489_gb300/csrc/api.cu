@@ -449,10 +449,17 @@ hr_status hr_create_scene(const hr_scene_desc* d, hr_scene* out) {
     };
     if (e != cudaSuccess) { delete s; return fail(HR_ERR_CUDA, "stream: %s", cudaGetErrorString(e)); }
     const size_t npx = (size_t)sc.W * sc.H * C;
-    // (a mesh has its target in tile order only: two copies of 786 KB each at 256x256
-    // made the allocator map another block per scene, a third of its creation)
-    const bool mesh = d->kind == HR_SCENE_REVOLVE3D;
-    if (!mesh && (e = cudaMalloc(&sc.target, sizeof(float) * npx)) != cudaSuccess) return bail(e, "target");
+    // One allocation for the target in all its orders: every further one of this size
+    // costs a creation 25 to 70 us.  Triangles: tile order | image.  (A mesh's stands below.)
+    const bool mesh = d->kind == HR_SCENE_REVOLVE3D, tris = d->kind == HR_SCENE_TRIS2D;
+    if (tris) {
+        const size_t tiled = tris2d_target_floats(sc);
+        if ((e = cudaMalloc(&sc.target4, sizeof(float) * (tiled + npx))) != cudaSuccess) return bail(e, "target");
+        sc.target = sc.target4 + tiled;
+    } else if (!mesh && (e = cudaMalloc(&sc.target, sizeof(float) * npx)) != cudaSuccess) {
+        return bail(e, "target");
+    }
+    float* mesh_image = nullptr;   // a caller's image, as it is given
     switch (d->kind) {
         case HR_SCENE_DISC2D: sc.radius = d->radius; break;
         case HR_SCENE_BOXES2D: sc.radius = d->radius; break;
@@ -471,11 +478,13 @@ hr_status hr_create_scene(const hr_scene_desc* d, hr_scene* out) {
             }
             if ((e = upload(&sc.verts, d->vertices, 3 * (size_t)sc.nv, s->stream)) != cudaSuccess) return bail(e, "vertices");
             if ((e = upload(&sc.tris, d->triangles, 3 * (size_t)sc.nt, s->stream)) != cudaSuccess) return bail(e, "triangles");
-            // one allocation: target in tile order | counters | sums by tile | normals
+            // one allocation: target in tile order | counters | sums by tile | normals | a caller's image
             const size_t tiles = revolve_tiles(sc), n_target = 3 * 8 * (size_t)sc.rv_th * tiles;
             const size_t n_stats = 8 * sizeof(unsigned long long) / sizeof(float);
-            if ((e = cudaMalloc(&sc.rv_target, sizeof(float) * (n_target + n_stats + tiles + 3 * (size_t)sc.nt))) != cudaSuccess)
+            const size_t n_tables = n_target + n_stats + tiles + 3 * (size_t)sc.nt;
+            if ((e = cudaMalloc(&sc.rv_target, sizeof(float) * (n_tables + (d->target_image ? npx : 0)))) != cudaSuccess)
                 return bail(e, "mesh tables");
+            mesh_image = sc.rv_target + n_tables;
             sc.rv_stats = reinterpret_cast<unsigned long long*>(sc.rv_target + n_target);
             sc.tile_t2 = sc.rv_target + n_target + n_stats;
             sc.tnrm = sc.tile_t2 + tiles;
@@ -518,12 +527,10 @@ hr_status hr_create_scene(const hr_scene_desc* d, hr_scene* out) {
         // no target: the loss is f itself
         if ((e = cudaMemsetAsync(sc.target, 0, sizeof(float) * npx, s->stream)) != cudaSuccess) return bail(e, "target");
     } else if (d->target_image && mesh) {
-        float* image = nullptr;
-        if ((e = upload(&image, d->target_image, npx, s->stream)) != cudaSuccess) return bail(e, "target upload");
-        revolve_tables(sc, image, s->stream);
-        e = cudaStreamSynchronize(s->stream);
-        cudaFree(image);
-        if (e != cudaSuccess) return bail(e, "target tiles");
+        if ((e = cudaMemcpyAsync(mesh_image, d->target_image, sizeof(float) * npx, cudaMemcpyHostToDevice, s->stream)) !=
+            cudaSuccess)
+            return bail(e, "target upload");
+        revolve_tables(sc, mesh_image, s->stream);
     } else if (d->target_image) {
         if ((e = cudaMemcpyAsync(sc.target, d->target_image, sizeof(float) * npx, cudaMemcpyHostToDevice, s->stream)) !=
             cudaSuccess)
@@ -543,8 +550,7 @@ hr_status hr_create_scene(const hr_scene_desc* d, hr_scene* out) {
         cudaFree(dp);
         if (e != cudaSuccess) return bail(e, "target render");
     }
-    if (sc.kind == HR_SCENE_TRIS2D && (e = tris2d_prepare_target(sc, s->stream)) != cudaSuccess)
-        return bail(e, "target tiles");
+    if (tris) tris2d_tile_target(sc, s->stream);
     if ((sc.kind == HR_SCENE_DISC2D || sc.kind == HR_SCENE_BOXES2D) &&
         (e = disc_prepare_target(sc, s->stream)) != cudaSuccess)
         return bail(e, "target bits");
@@ -558,9 +564,10 @@ hr_status hr_destroy_scene(hr_scene s) {
     if (!s) return HR_OK;
     DevScene& sc = s->sc;
     if (s->stream) cudaStreamSynchronize(s->stream);
-    cudaFree(sc.target); cudaFree(sc.verts); cudaFree(sc.tris);
+    cudaFree(sc.target4 ? sc.target4 : sc.target);   // (one allocation)
+    cudaFree(sc.verts); cudaFree(sc.tris);
     cudaFree(sc.rv_target);   // (holds the other mesh tables)
-    cudaFree(sc.raw); cudaFree(sc.pidx); cudaFree(sc.target4); cudaFree(sc.qA); cudaFree(sc.qb);
+    cudaFree(sc.raw); cudaFree(sc.pidx); cudaFree(sc.qA); cudaFree(sc.qb);
     cudaFree(sc.pt_stats); cudaFree(sc.tbits);   // (holds the other target tables)
     s->ws.release_all();
     for (cudaEvent_t& e : s->ev)

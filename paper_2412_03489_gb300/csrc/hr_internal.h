@@ -265,7 +265,8 @@ void launch_revolve_target(const DevScene& sc, const float* params, cudaStream_t
 // the sums by tile, and before them rv_target from an image [H][W][3] if one is given
 void revolve_tables(DevScene& sc, const float* image, cudaStream_t s);
 cudaError_t ptbox_prepare();   // kernel attributes
-cudaError_t tris2d_prepare_target(DevScene& sc, cudaStream_t s);   // after the target exists: sc.target4
+size_t tris2d_target_floats(const DevScene& sc);   // of sc.target4
+void tris2d_tile_target(const DevScene& sc, cudaStream_t s);   // after the target exists: sc.target4 from it
 // disc and squares scenes, after the target exists: sc.tbits, sc.tbinary, sc.tones and (disc) sc.tpre, sc.centres
 cudaError_t disc_prepare_target(DevScene& sc, cudaStream_t s);
 

@@ -383,13 +383,14 @@ void launch_tris2d_loss(const DevScene& sc, const RenderBatch& b, cudaStream_t s
     else launch_loss<1>(sc, b, s);
 }
 
-cudaError_t tris2d_prepare_target(DevScene& sc, cudaStream_t s) {
+size_t tris2d_target_floats(const DevScene& sc) {
+    return 4 * 32 * (size_t)((sc.W + 7) / 8) * ((sc.H + 3) / 4);
+}
+
+void tris2d_tile_target(const DevScene& sc, cudaStream_t s) {
     const int TXn = (sc.W + 7) / 8, n = 32 * TXn * ((sc.H + 3) / 4);
-    const cudaError_t e = cudaMalloc((void**)&sc.target4, sizeof(float4) * (size_t)n);
-    if (e != cudaSuccess) return e;
     tris2d_target_kernel<<<(n + 255) / 256, 256, 0, s>>>(sc.target, sc.W, sc.H, TXn, n,
                                                          reinterpret_cast<float4*>(sc.target4));
-    return cudaGetLastError();
 }
 
 void launch_tris2d_image(const DevScene& sc, const float* params, float* img, cudaStream_t s) {
