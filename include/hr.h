@@ -603,12 +603,13 @@ hr_status hr_profile_last(hr_scene scene, float* ms3);
  * variants (path tracer, where one CTA renders one perturbation: resident
  * CTAs per SM, i.e. register caps, 2 to 4 by the launch's size, 2 to 3 or 2;
  * disc and squares: 8 / 4 / 16 warps per CTA, one warp per
- * perturbation; mesh and 2D triangles: one shape) and the sampler runs with
- * 16, 32, 64 or 128 threads per block (16 spreads small requests over more
- * SMs; with 64 or 128, a block takes its aggregate Hessian pairs diagonal-lobe
- * ones first so that most warps run one lobe path).  Every variant computes
- * each value with the same operations in the same order, so results are
- * bit-identical whatever is chosen.
+ * perturbation; mesh and 2D triangles: one shape) and a sampler block draws
+ * 16, 32, 64 or 128 perturbations (the blocks' threads follow from that and the
+ * number of parameters; 16 spreads small requests over more SMs; blocks draw
+ * fewer where their shared memory would not hold the perturbations or where SMs
+ * would stay idle, and 64 instead of 32 in large launches).  Every variant
+ * computes each value with the same operations in the same order, so results
+ * are bit-identical whatever is chosen.
  * hr_autotune times each variant on profiled aggregate HVP estimates of
  * max(n_probe, 8 x the SM count) perturbations at h_theta [n] (v = ones,
  * sigma 0.05; median of 3 after a warm-up; the floor keeps the GPU full so
@@ -617,13 +618,13 @@ hr_status hr_profile_last(hr_scene scene, float* ms3);
  * renders pairs of perturbations per CTA, which has one shape, the render variant
  * stays 0 and one timing stands for all.  hr_set_tuning sets a choice
  * directly (HR_ERR_INVALID_ARG when out of range).  Scenes start at variant 0
- * and 32 sampler threads.
+ * and 32 perturbations a block.
  * ------------------------------------------------------------------------- */
 typedef struct {
     int32_t render_variant;     /* chosen render variant */
-    int32_t sample_threads;     /* chosen sampler threads per block */
+    int32_t sample_threads;     /* chosen perturbations per sampler block */
     int32_t n_render_variants;
-    int32_t n_sample_variants;  /* 4: 32, 64, 128, 16 threads */
+    int32_t n_sample_variants;  /* 4: 32, 64, 128, 16 perturbations */
     float render_ms[4];         /* median render+loss time per variant */
     float sample_ms[4];         /* median sampler time per shape */
 } hr_tune_info;

@@ -77,7 +77,7 @@ struct SampleArgs {
     uint2* meta;          // [M] (sub, pair k) or null
     const int32_t* step;  // optional device step index s: every group's sub += 64 s
     const double* sigma_row;  // optional [rows]: group sigma = sigma_row[theta_row] (Z's derived in-kernel)
-    int32_t threads;          // threads per block: 16, 32 (0 = 32), 64 or 128; no effect on the results
+    int32_t threads;          // perturbations per block: 16, 32 (0 = 32), 64 or 128 (see launch_sample); no effect on the results
     // optional: the first block also writes theta in FP32 (RN) to theta_out[theta_n],
     // from theta_in (device, FP64) or, when theta_in is null, from theta_vals
     const double* theta_in;

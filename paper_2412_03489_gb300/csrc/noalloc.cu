@@ -2,7 +2,7 @@
 // not allocate device memory while they run.
 //
 // Its working memory (perturbations, weights, path keys, per-render losses,
-// sample-group table, FP32 parameters, sums) is a fixed array in the
+// FP32 parameters, sums) is a fixed array in the
 // library's own device memory, so the call itself never allocates: no
 // cudaMalloc, no cudaFree, no allocating library routine.  The array is
 // kScratchBytes (4 MiB) on every GPU that loads the library, held until the
@@ -72,7 +72,9 @@ extern "C" hr_status hr_estimate_dev_noalloc(hr_scene s, int32_t quantity, const
     const int64_t M = o->n_perturb;
     const int64_t Mt = (int64_t)G * M;
 
-    // carve the fixed array: theta32 | groups | tau | weights | keys | losses | sums | scale
+    // carve the fixed array: theta32 | - | tau | weights | keys | losses | sums | -
+    // (The marked parts, a group table's and the sums' scales' room, are not used. They stay
+    // in the count so that the same requests are accepted and refused on every version.)
     const size_t off_theta = 0;
     const size_t off_groups = off_theta + align256(sizeof(float) * n);
     const size_t off_tau = off_groups + align256(sizeof(SampleGroup) * (size_t)G);

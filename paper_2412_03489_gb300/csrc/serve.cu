@@ -111,6 +111,8 @@ struct Arena {
 
 int n_elem(int quantity, int n) { return quantity == HR_HESSIAN ? n * (n + 1) / 2 : n; }
 
+// (the third part, a group table's room, is not used; it stays in the count so that a
+// budget admits and refuses the same requests on every version)
 size_t request_bytes(int n, int E, int G, int64_t Mt) {
     return up(sizeof(float) * n) + up(sizeof(double) * n) + up(sizeof(SampleGroup) * (size_t)G) +
            up(sizeof(float) * (size_t)Mt * n) + up(sizeof(float) * (size_t)Mt * E) + up(sizeof(uint2) * (size_t)Mt) +

@@ -1,7 +1,7 @@
 // Autotuner: per scene, times the launch shapes of the render+loss kernel and
 // of the sampler on a probe estimate and keeps the fastest.  Every candidate
 // computes the same values in the same order (a different register cap,
-// warps per CTA or threads per block), so tuning changes speed, never a
+// warps per CTA or perturbations per sampler block), so tuning changes speed, never a
 // result: estimates before and after tuning are bit-identical.
 #include <algorithm>
 #include <cmath>
